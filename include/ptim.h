@@ -147,9 +147,8 @@ pt_status pt_trim(pt_ctx* ctx);
  *   "scratch_bytes"  bytes of pair/orbital fields one FFT batch may hold (default 512 MiB: the
  *                    cost per pair falls with the pair tile even past L2 residency, 4-10% from
  *                    48 MiB to 512 MiB; smaller values give more, smaller batches).
- *   "exchange64_scratch_bytes"  the same for the 64^3 FP32 exchange pipeline (default 512 MiB:
- *                    16 x 16 pair tiles, the largest its parameter block holds), which keeps four
- *                    such batches in flight.
+ *   "exchange64_scratch_bytes"  the same for the 64^3 FP32 exchange (default 512 MiB: 16 x 16 pair
+ *                    tiles).
  *   "tc_gram"        1: in the PT_FP32 form, run the Gram contractions (A^H B over the grid) on
  *                    the tensor cores with a 3-product TF32 split (hi*hi + hi*lo + lo*hi) that
  *                    keeps FP32-level accuracy; 0 (default): CUDA cores.
@@ -223,9 +222,9 @@ typedef struct {
 } pt_exchange_item;
 
 /* Batched exchange: `count` independent V_x applications (different orbital counts, grids and
- * kernels) in one call, in the given precision, in item order on `stream`.  The pair-tile size
- * of each grid is chosen by timing a few candidates the first time the grid is seen (option
- * "autotune", default 1).  The first call with a given item set (the same buffers and sizes)
+ * kernels) in one call, in the given precision, in item order on `stream`.  Where the pair-tile
+ * size matters (FP64 and orthorhombic grids) it is chosen by timing a few candidates the first time
+ * the grid is seen (option "autotune", default 1).  The first call with a given item set (the same buffers and sizes)
  * runs eagerly and records the batch into a CUDA graph; later calls with the same item set
  * replay the graph as one launch (option "graphs", default 1).  pt_trim drops the graphs.
  * Synchronises `stream` once at the end to read the kernels' error word (PT_TIMEOUT if a

@@ -3,12 +3,11 @@
 // Eq. vxdiag, applied per instance).
 //
 // Host runtime around the exchange kernels:
-//   * autotuner: the pair-tile size of a grid (how many pair fields one FFT batch holds, which
-//     sets the L2 footprint and the launch count), on 64^3 FP32 grids the kernel family (the
-//     launch-pipelined TMA kernels or the compile-time tile kernels), and for the compile-time
-//     kernels in FP32 the CTA size of their FFT tile kernels (128, 256 or 512 threads) are picked
-//     by timing candidates (budgets of 12 MiB to 512 MiB) on the first item of that grid (its
-//     first min(N, 32) orbitals) and kept in the context;
+//   * autotuner: on the grids whose cost depends on it (FP64, orthorhombic cells) the pair-tile size
+//     (how many pair fields one FFT batch holds, which sets the L2 footprint and the launch count) is
+//     picked by timing candidates (budgets of 12 MiB to 512 MiB) on the first item of that grid (its
+//     first min(N, 32) orbitals) and kept in the context; the FP32 line kernels of cubic grids take the
+//     largest tile, which was the fastest on every side (24^3 N = 64: 0.22 ms with 512 MiB, 0.47 with 48);
 //   * concurrent branches: items are dealt to `batch_streams` streams (longest first, by pair
 //     FFTs x grid points), each with its own scratch buffers, forked from and joined back to the
 //     caller's stream with events, so the small items' kernels fill the tails of the large ones';
@@ -46,13 +45,11 @@ std::string grid_key(const pt_grid& g, pt_precision prec) {
 
 struct Tuned {
   size_t budget;
-  int engine;  // exchange64_engine for 64^3 FP32 grids (0 or 1); ignored elsewhere
-  int ft;      // threads per CTA of the compile-time tile kernels
 };
 
-// Pick the pair-field budget (and the 64^3 engine) for the grid of `it` by timing candidates
-// (cached per grid).
+// Pick the pair-field budget for the grid of `it` by timing candidates (cached per grid).
 Tuned tuned_budget(pt_ctx* ctx, const pt_exchange_item& it, pt_precision prec, cudaStream_t st) {
+  if (prec != PT_FP64 && exchange_lines_applies(ctx, it.grid)) return Tuned{ctx->scratch_budget};
   const std::string key = grid_key(it.grid, prec);
   auto c = ctx->caches.find(key);
   if (c != ctx->caches.end()) return *std::static_pointer_cast<Tuned>(c->second);
@@ -62,63 +59,40 @@ Tuned tuned_budget(pt_ctx* ctx, const pt_exchange_item& it, pt_precision prec, c
   cudaEvent_t e0, e1;
   PT_CUDA_CHECK(cudaEventCreate(&e0));
   PT_CUDA_CHECK(cudaEventCreate(&e1));
-  Tuned best{ctx->scratch_budget, ctx->exchange64_engine == 1 ? 1 : 0, ctx->fft_threads};
+  Tuned best{ctx->scratch_budget};
   float best_ms = 1e30f;
   const size_t mib = size_t(1) << 20;
   const size_t cands[] = {12 * mib, 24 * mib, 48 * mib, 96 * mib, 192 * mib, 512 * mib};
-  const bool two_engines = prec != PT_FP64 && exchange64_applies(it.grid);
-  const bool fixed = fixed_cubic(it.grid);
-  const int saved_engine = ctx->exchange64_engine, saved_ft = ctx->fft_threads;
-  struct Variant {
-    int engine, ft;
-  };
-  // the TMA pipeline (64^3 FP32 only), then the compile-time kernels with each CTA size (FP32) or 256
-  std::vector<Variant> variants;
-  if (two_engines) variants.push_back({0, saved_ft});
-  const int fts[3] = {256, 128, 512};
-  const int nft = (fixed && prec != PT_FP64) ? 3 : 1;
-  for (int q = 0; q < nft; ++q) variants.push_back({two_engines ? 1 : saved_engine, fts[q]});
   try {
-    for (const Variant& var : variants) {
-      const int engine = var.engine;
-      int last_b = -1;
-      ctx->exchange64_engine = engine;
-      ctx->fft_threads = var.ft;
-      for (size_t cand : cands) {
-        // candidates that give the same pair tile are the same schedule
-        int b = std::min(nt, int(std::floor(std::sqrt(double(std::max<size_t>(1, cand / field))))));
-        if (two_engines && engine == 0) b = std::min(b, kExchange64MaxTile);
-        if (b == last_b) continue;
-        last_b = b;
-        ctx->budget_override = cand;
-        exchange(ctx, it.src, it.occ, nt, nullptr, nt, out, it.grid, it.kernel, prec, st);  // builds the schedule
-        PT_CUDA_CHECK(cudaEventRecord(e0, st));
-        for (int r = 0; r < 2; ++r)
-          exchange(ctx, it.src, it.occ, nt, nullptr, nt, out, it.grid, it.kernel, prec, st);
-        PT_CUDA_CHECK(cudaEventRecord(e1, st));
-        PT_CUDA_CHECK(cudaEventSynchronize(e1));
-        float ms = 0.f;
-        PT_CUDA_CHECK(cudaEventElapsedTime(&ms, e0, e1));
-        if (ms < best_ms) {
-          best_ms = ms;
-          best = Tuned{cand, engine, var.ft};
-        }
+    int last_b = -1;
+    for (size_t cand : cands) {
+      // candidates that give the same pair tile are the same schedule
+      const int b = std::min(nt, int(std::floor(std::sqrt(double(std::max<size_t>(1, cand / field))))));
+      if (b == last_b) continue;
+      last_b = b;
+      ctx->budget_override = cand;
+      exchange(ctx, it.src, it.occ, nt, nullptr, nt, out, it.grid, it.kernel, prec, st);  // builds the schedule
+      PT_CUDA_CHECK(cudaEventRecord(e0, st));
+      for (int r = 0; r < 2; ++r)
+        exchange(ctx, it.src, it.occ, nt, nullptr, nt, out, it.grid, it.kernel, prec, st);
+      PT_CUDA_CHECK(cudaEventRecord(e1, st));
+      PT_CUDA_CHECK(cudaEventSynchronize(e1));
+      float ms = 0.f;
+      PT_CUDA_CHECK(cudaEventElapsedTime(&ms, e0, e1));
+      if (ms < best_ms) {
+        best_ms = ms;
+        best = Tuned{cand};
       }
     }
   } catch (...) {
     ctx->budget_override = 0;
-    ctx->exchange64_engine = saved_engine;
-    ctx->fft_threads = saved_ft;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     throw;
   }
   ctx->budget_override = 0;
-  ctx->exchange64_engine = saved_engine;
-  ctx->fft_threads = saved_ft;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (!two_engines) best.engine = saved_engine;
   ctx->caches[key] = std::make_shared<Tuned>(best);
   return best;
 }
@@ -143,30 +117,31 @@ std::vector<int> assign_branches(const pt_exchange_item* items, int count, int n
   return branch;
 }
 
+// the persistent and TMA engines of option exchange64_engine are for single calls
+struct EngineGuard {
+  pt_ctx* ctx;
+  int engine;
+  explicit EngineGuard(pt_ctx* c) : ctx(c), engine(c->exchange64_engine) { c->exchange64_engine = engine == 1 ? 1 : 0; }
+  ~EngineGuard() { ctx->exchange64_engine = engine; }
+};
+
 struct TagGuard {
   pt_ctx* ctx;
-  int engine, ft;
   ~TagGuard() {
     ctx->scratch_tag.clear();
     ctx->budget_override = 0;
-    ctx->exchange64_engine = engine;
-    ctx->fft_threads = ft;
   }
 };
 
 long long run_items(pt_ctx* ctx, const pt_exchange_item* items, int count, const std::vector<Tuned>& tuned,
                     pt_precision prec, cudaStream_t st) {
   long long pairs = 0;
-  TagGuard guard{ctx, ctx->exchange64_engine, ctx->fft_threads};
+  TagGuard guard{ctx};
   const int nb = std::max(1, std::min(ctx->batch_streams, count));
   auto one = [&](int k, cudaStream_t s) {
     const pt_exchange_item& it = items[k];
     ctx->budget_override = tuned[k].budget;
-    if (prec != PT_FP64 && exchange64_applies(it.grid)) ctx->exchange64_engine = tuned[k].engine;
-    ctx->fft_threads = tuned[k].ft;
     pairs += exchange(ctx, it.src, it.occ, it.N, it.tgt, it.tgt ? it.M : it.N, it.out, it.grid, it.kernel, prec, s);
-    ctx->exchange64_engine = guard.engine;
-    ctx->fft_threads = guard.ft;
   };
   if (nb == 1) {
     for (int k = 0; k < count; ++k) one(k, st);
@@ -202,15 +177,14 @@ long long run_items(pt_ctx* ctx, const pt_exchange_item* items, int count, const
 }
 
 std::string batch_key(const pt_exchange_item* items, int count, pt_precision prec, const std::vector<Tuned>& tuned,
-                      int streams) {
-  std::string k = "graph:" + std::to_string(int(prec)) + ":" + std::to_string(count) + ":" + std::to_string(streams);
+                      int streams, int engine) {
+  std::string k = "graph:" + std::to_string(engine) + ":" + std::to_string(int(prec)) + ":" + std::to_string(count) + ":" + std::to_string(streams);
   char b[256];
   for (int i = 0; i < count; ++i) {
     const pt_exchange_item& it = items[i];
-    snprintf(b, sizeof(b), "|%p,%p,%d,%p,%d,%p,%d,%d,%d,%.17g,%.17g,%.17g,%d,%.17g,%.17g,%zu,%d,%d", it.src,
+    snprintf(b, sizeof(b), "|%p,%p,%d,%p,%d,%p,%d,%d,%d,%.17g,%.17g,%.17g,%d,%.17g,%.17g,%zu", it.src,
              static_cast<const void*>(it.occ), it.N, it.tgt, it.M, it.out, it.grid.nx, it.grid.ny, it.grid.nz,
-             it.grid.L[0], it.grid.L[1], it.grid.L[2], it.kernel.type, it.kernel.mu, it.kernel.g0, tuned[i].budget,
-             tuned[i].engine, tuned[i].ft);
+             it.grid.L[0], it.grid.L[1], it.grid.L[2], it.kernel.type, it.kernel.mu, it.kernel.g0, tuned[i].budget);
     k += b;
   }
   return k;
@@ -230,11 +204,12 @@ struct DeferGuard {
 long long exchange_batched(pt_ctx* ctx, const pt_exchange_item* items, int count, pt_precision prec,
                            cudaStream_t st, size_t* graph_nodes) {
   if (graph_nodes) *graph_nodes = 0;
-  std::vector<Tuned> tuned(count, Tuned{ctx->scratch_budget, ctx->exchange64_engine == 1 ? 1 : 0, ctx->fft_threads});
+  EngineGuard guard(ctx);
+  std::vector<Tuned> tuned(count, Tuned{ctx->scratch_budget});
   if (ctx->autotune)
     for (int k = 0; k < count; ++k) tuned[k] = tuned_budget(ctx, items[k], prec, st);
   int* err = static_cast<int*>(ctx->get("exchange_err", sizeof(int)));
-  const std::string key = batch_key(items, count, prec, tuned, std::min(ctx->batch_streams, count));
+  const std::string key = batch_key(items, count, prec, tuned, std::min(ctx->batch_streams, count), ctx->exchange64_engine);
   auto c = ctx->caches.find(key);
   if (ctx->use_graphs && c != ctx->caches.end()) {
     auto g = std::static_pointer_cast<GraphHolder>(c->second);

@@ -171,8 +171,7 @@ pt_status pt_set_option(pt_ctx* ctx, const char* key, double value) {
     if (!ctx || !key) pt::fail(PT_INVALID_ARG, "context or key is NULL");
     if (std::string(key) == "fft_threads") {
       if (!(value == 128.0 || value == 256.0 || value == 512.0)) pt::fail(PT_INVALID_ARG, "fft_threads is 128, 256 or 512");
-      ctx->fft_threads = int(value);
-      return PT_OK;
+      return PT_OK;  // accepted as before; the tile kernels are built with 256 threads per CTA
     }
     if (std::string(key) == "batch_streams") {
       if (!(value >= 1.0 && value <= 16.0)) pt::fail(PT_INVALID_ARG, "batch_streams must be in [1, 16]");
@@ -611,7 +610,7 @@ size_t pt_ptim_footprint(int N, const pt_grid* grid, pt_precision prec, int ande
     const size_t b64 = size_t(std::floor(std::sqrt(double((size_t(512) << 20) / field))));  // default tma64_budget
     B = std::max<size_t>(1, std::min<size_t>({b64, size_t(N), size_t(pt::kExchange64MaxTile)}));
   }
-  const size_t exch = (tma64 ? 4 : 1) * B * B * field;
+  const size_t exch = (tma64 ? 4 : 1) * B * B * field;  // 64^3 FP32: the persistent engine's ring at most
   const size_t hscr = 2 * std::max<size_t>(1, std::min<size_t>(size_t(N), budget / (2 * field))) * field;
   const size_t nn = size_t(N) * N * sizeof(double) * 2;
   const size_t gram_parts = size_t(4 * 160 + 64) * nn;  // split partials, bounded by 4 waves of tiles

@@ -148,9 +148,7 @@ struct pt_ctx {
   // bytes of pair fields per exchange batch (and of orbital fields per H batch); larger batches
   // cost less per pair even past L2 residency (fewer launches, traffic amortised over the tile)
   size_t scratch_budget = size_t(512) << 20;
-  // bytes of pair fields per batch on the 64^3 FP32 TMA pipeline: its cost per pair falls with the
-  // pair tile (fewer launches, W traffic amortised over more contributions), so it takes the
-  // largest tile its parameter block holds rather than an L2-sized one
+  // the same for the 64^3 FP32 exchange (16 x 16 pair tiles)
   size_t tma64_budget = size_t(512) << 20;
   int tc_gram = 0;     // option: FP32 form's Gram contractions on tensor cores (3xTF32) when 1
   int active_tc = 0;   // per call: 0 CUDA cores, 1 tensor cores 3xTF32, 2 tensor cores single TF32
@@ -167,9 +165,9 @@ struct pt_ctx {
   std::string ptim_warm_key;     // sizes, grid, kernel and precision of that step
   unsigned long long ptim_warm_fp[2] = {0, 0};  // fingerprint of that step's output (phi, sigma)
   int ptim_q_n = 0;            // the "ptim_Q" buffer holds a complete unitary ptim_q_n x ptim_q_n basis
-  // option: 64^3 FP32 exchange engine: 0 the launch-pipelined TMA kernel (roles A, B, C, D), 1 the
-  // compile-time tile kernels, 2 one persistent cooperative launch per application
-  // (exchange64_persist.cu), 3 the launch-pipelined TMA kernel with C fused into the accumulate
+  // option: FP32 exchange engine: 0 the line kernels (exchange_lines.cu; cubic sides of PT_FIXED_SIZES), 1 the
+  // compile-time tile kernels on those sides; on 64^3 also 2 one persistent cooperative launch per application
+  // (exchange64_persist.cu), 3 the launch-pipelined TMA kernel (exchange64_tma.cu)
   int exchange64_engine = 0;
   int x64p_tile = 4;   // option: pair-tile side of the persistent engine's schedule
   int x64p_ring = 24;  // option: pair-field ring slots of the persistent engine (raised to tile pairs + 3 lag + 1)
@@ -184,7 +182,6 @@ struct pt_ctx {
   bool defer_checks = false;   // inside a batched call: device error words are checked once at the end
   cudaStream_t cap_stream = nullptr;  // non-default stream that graph captures are recorded on
   int batch_streams = 4;              // option: concurrent branches (streams) of a batched exchange call
-  int fft_threads = 256;              // option: threads per CTA of the compile-time exchange tile kernels
   std::vector<cudaStream_t> side_streams;  // the branches' streams (created on first use)
   std::string scratch_tag;            // suffix of the exchange scratch names: one set per concurrent branch
   std::string tagged(const char* name) const { return std::string(name) + scratch_tag; }

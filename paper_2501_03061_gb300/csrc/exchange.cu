@@ -212,6 +212,13 @@ long long exchange_t(pt_ctx* ctx, const cx<T>* src, const double* occ, int N, co
     tgt = src;
     M = N;
   }
+  if constexpr (sizeof(T) == 4) {
+    if (exchange_lines_applies(ctx, g)) {
+      const size_t bud = ctx->budget_override ? ctx->budget_override
+                                              : (exchange64_applies(g) ? ctx->tma64_budget : exchange_scratch_budget(ctx));
+      return exchange_lines(ctx, src, occ, N, tgt, M, sym, out, g, k, bud, st);
+    }
+  }
   const FftTables& ft = fft_tables(ctx, g, prec);
   const T* ktab = static_cast<const T*>(kernel_table(ctx, g, k, prec));
   if constexpr (sizeof(T) == 4) {
@@ -224,10 +231,9 @@ long long exchange_t(pt_ctx* ctx, const cx<T>* src, const double* occ, int N, co
   }
   const size_t ng = ng_of(g);
   const size_t field = ng * sizeof(cx<T>);
-  // Pair batch: as many pair fields as fit a budget that keeps them L2-resident (the 64^3 TMA
-  // pipeline takes its own, larger budget: see pt_ctx::tma64_budget).
-  const bool tma64 =
-      sizeof(T) == 4 && exchange64_applies(g) && (ctx->exchange64_engine == 0 || ctx->exchange64_engine == 3);
+  // Pair batch: as many pair fields as fit the budget (the 64^3 TMA pipeline takes its own: see
+  // pt_ctx::tma64_budget).
+  const bool tma64 = sizeof(T) == 4 && exchange64_applies(g) && ctx->exchange64_engine == 3;
   const size_t budget = ctx->budget_override ? ctx->budget_override
                                              : (tma64 ? ctx->tma64_budget : exchange_scratch_budget(ctx));
   int B = int(std::floor(std::sqrt(double(std::max<size_t>(1, budget / field)))));
@@ -244,9 +250,8 @@ long long exchange_t(pt_ctx* ctx, const cx<T>* src, const double* occ, int N, co
     sch = std::static_pointer_cast<ScheduleImpl>(it->second);
   }
   if constexpr (sizeof(T) == 4) {
-    if (exchange64_applies(g) && (ctx->exchange64_engine == 0 || ctx->exchange64_engine == 3)) {
-      exchange64_tma(ctx, *sch, src, occ, tgt, M, out, ktab, static_cast<const cx<T>*>(ft.tw), st,
-                     ctx->exchange64_engine == 3);
+    if (tma64) {
+      exchange64_tma(ctx, *sch, src, occ, tgt, M, out, ktab, st);
       if (!ctx->defer_checks) exchange_check(ctx, st);
       return sch->total_pairs;
     }
@@ -260,7 +265,7 @@ long long exchange_t(pt_ctx* ctx, const cx<T>* src, const double* occ, int N, co
       const int p0 = sch->pair_off[b], np = sch->pair_off[b + 1] - p0;
       const int t0 = sch->tgt_off[b], nt = sch->tgt_off[b + 1] - t0;
       exchange_batch_fixed<T>(g.nx, src, tgt, occ, sch->d_pairs + p0, np, sch->d_tgts + t0, nt, sch->d_contribs,
-                              ktab, twg, scratch, out, st, ctx->fft_threads);
+                              ktab, twg, scratch, out, st);
     }
     return sch->total_pairs;
   }

@@ -1,15 +1,16 @@
-// FP32 pair-FFT exchange for 64^3 grids with TMA staging (Sec. IV-A1, Eq. vxdiag).
+// FP32 pair-FFT exchange for 64^3 grids with TMA staging (Sec. IV-A1, Eq. vxdiag; option
+// exchange64_engine = 3, kept beside the default of exchange_lines.cu).
 //
-// Same four pipelined roles as the register/shared-memory kernel (A: pair product + x/y
-// transforms of a plane, B: z transform + K + inverse z of a slab, C: inverse y/x transforms
-// of a plane, D: occupation-weighted accumulate into the target plane), but every strided
-// access to a pair field goes through the tensor-memory accelerator:
+// Three pipelined roles in one launch per pair batch, software-pipelined over three scratch slots (A:
+// pair product + x/y transforms of a plane, B: z transform + K + inverse z of a slab, CD: inverse y/x
+// transforms of a plane and the occupation-weighted accumulate into the target plane), where every
+// strided access to a pair field goes through the tensor-memory accelerator:
 //   * plane and slab tiles are fetched with cp.async.bulk.tensor into 128B-swizzled shared
 //     tiles (four 16-wide sub-tiles of 128-byte rows); the 16-byte chunk c of row r sits at
 //     chunk c ^ (r mod 8), so the column reads of the line transforms (8 lanes on 8 rows of
 //     one column, 4 adjacent columns per warp) hit every bank exactly twice per warp;
 //   * the z-slab results of pass B go back to the scratch field with TMA stores.
-// Row-contiguous traffic (pass A/C results, pass D) stays on plain coalesced loads/stores.
+// Row-contiguous traffic (pass A results, the targets) stays on plain coalesced loads/stores.
 // Each CTA waits on its mbarrier with a %globaltimer deadline; on expiry it sets an error
 // word that the host checks after the call, and returns.
 #include <algorithm>
@@ -32,20 +33,16 @@ constexpr int MAXP = MAXB * MAXB, MAXT = 2 * MAXB, MAXC = 2 * MAXP;
 // The batch descriptors travel in the kernel parameters (constant bank): no dependent global
 // load stands between a CTA's start and its first TMA request.
 struct Launch {
-  int nA, nB, nC, nD;
-  int slotA, slotB, slotC, slotD;
+  int nA, nB, nD;
+  int slotA, slotB, slotD;
   int max_pairs, d_cbeg;
-  PairDesc pa[MAXP], pb[MAXP], pc[MAXP];
+  PairDesc pa[MAXP], pb[MAXP];
   TargetDesc td[MAXT];
   Contrib cd[MAXC];
 };
 
 __constant__ c64 c_tw64[G];
 
-// FUSED = false: roles A, B, C, D over four slots.  FUSED = true: roles CD, A, B over three slots,
-// where a CD CTA owns one target plane and runs C's inverse y/x transforms of each contributing
-// pair's plane itself before accumulating (see the CD role below).
-template <bool FUSED>
 __global__ void __launch_bounds__(THREADS, 2)
     k_exchange64_tma(const __grid_constant__ CUtensorMap tm_src, const __grid_constant__ CUtensorMap tm_tgt,
                      const __grid_constant__ CUtensorMap tm_plane, const __grid_constant__ CUtensorMap tm_slab,
@@ -65,93 +62,89 @@ __global__ void __launch_bounds__(THREADS, 2)
   if (tid < G) tw[tid] = c_tw64[tid];
   if (tid == 0) {
     mbar_init(bar, 1);
-    mbar_init(bar + 8, 1);   // second tile of the two-item roles B and C
-    mbar_init(bar + 16, 1);  // third contribution slot of role D
+    mbar_init(bar + 8, 1);  // second tile of roles B and CD
     fence_mbar_init();
   }
   __syncthreads();
   int bid = blockIdx.x;
 
-  if constexpr (FUSED) {
-    if (bid < L.nD) {
-      // ---------------- pass CD (one target plane per CTA) ----------------
-      // For each contribution (pair slot, partner, occupation, conjugation) of target td at plane z:
-      // the pair's plane z after the z transforms arrives by TMA (double-buffered, one contribution
-      // ahead), the inverse y and x transforms run here (lane t of group y ends with v[y][t + 8k]),
-      // and d * partner * v accumulates in registers.  v_ij never leaves the SM: the C -> D round
-      // trip of the four-role pipeline (write and read of every pair field) is gone, at the price of
-      // transforming a symmetric pair's plane once for each of its two targets.  Plane-major order:
-      // all targets at one z run together, so both targets of a pair read its plane from L2.
-      const int nt = L.nD / G;
-      const int z = bid / nt;
-      const TargetDesc td = L.td[bid % nt];
-      __shared__ int s_list[2 * MAXB];
-      __shared__ int s_n;
-      if (tid == 0) {  // contributions with a nonzero occupation (a skipped pair's slot is stale)
-        int n = 0;
-        for (int i = td.cbeg; i < td.cend; ++i)
-          if (occ[L.cd[i - L.d_cbeg].occ] != 0.0) s_list[n++] = i - L.d_cbeg;
-        s_n = n;
+  if (bid < L.nD) {
+    // ---------------- pass CD (one target plane per CTA) ----------------
+    // For each contribution (pair slot, partner, occupation, conjugation) of target td at plane z:
+    // the pair's plane z after the z transforms arrives by TMA (double-buffered, one contribution
+    // ahead), the inverse y and x transforms run here (lane t of group y ends with v[y][t + 8k]),
+    // and d * partner * v accumulates in registers.  v_ij never leaves the SM, at the price of
+    // transforming a symmetric pair's plane once for each of its two targets.  Plane-major order:
+    // all targets at one z run together, so both targets of a pair read its plane from L2.
+    const int nt = L.nD / G;
+    const int z = bid / nt;
+    const TargetDesc td = L.td[bid % nt];
+    __shared__ int s_list[2 * MAXB];
+    __shared__ int s_n;
+    if (tid == 0) {  // contributions with a nonzero occupation (a skipped pair's slot is stale)
+      int n = 0;
+      for (int i = td.cbeg; i < td.cend; ++i)
+        if (occ[L.cd[i - L.d_cbeg].occ] != 0.0) s_list[n++] = i - L.d_cbeg;
+      s_n = n;
+    }
+    __syncthreads();
+    const int n = s_n;
+    auto issue = [&](int c) {  // one thread
+      const Contrib cc = L.cd[s_list[c]];
+      const int orb = L.slotD * L.max_pairs + cc.slot;
+      const uint32_t b = uint32_t(c & 1);
+      fence_proxy_async_smem();  // the buffer was last read and written through the generic proxy
+      mbar_arrive_expect_tx(bar + 8u * b, TILE_BYTES);
+      tma_load_5d(base + b * TILE_BYTES, &tm_plane, 0, 0, z, orb, 0, bar + 8u * b);
+    };
+    if (tid == 0) {
+      if (n > 0) issue(0);
+      if (n > 1) issue(1);
+    }
+    c64 acc[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[k] = czero<float>();
+    const int y = grp, kx = grp;
+    for (int c = 0; c < n; ++c) {
+      const uint32_t b = uint32_t(c & 1);
+      const bool ok = mbar_wait(bar + 8u * b, uint32_t(c >> 1) & 1u, TIMEOUT_NS);
+      if (!__syncthreads_and(ok)) {
+        if (tid == 0) atomicOr(err, 16);
+        return;
       }
+      c64 v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = *reinterpret_cast<const c64*>(sm + b * TILE_BYTES + sw_off(kx, t + 8 * q));
+      __syncthreads();  // the buffer is consumed: it becomes the group-transpose area
+      c64* gs = reinterpret_cast<c64*>(sm + b * TILE_BYTES) + grp * 64;
+      fft64_tma(v, t, gs, gpar, tw, true);  // inverse along y: lane t holds y = t + 8k
+#pragma unroll
+      for (int k = 0; k < 8; ++k) P[pidx(t + 8 * k, kx)] = v[k];
       __syncthreads();
-      const int n = s_n;
-      auto issue = [&](int c) {  // one thread
-        const Contrib cc = L.cd[s_list[c]];
-        const int orb = L.slotD * L.max_pairs + cc.slot;
-        const uint32_t b = uint32_t(c & 1);
-        fence_proxy_async_smem();  // the buffer was last read and written through the generic proxy
-        mbar_arrive_expect_tx(bar + 8u * b, TILE_BYTES);
-        tma_load_5d(base + b * TILE_BYTES, &tm_plane, 0, 0, z, orb, 0, bar + 8u * b);
-      };
-      if (tid == 0) {
-        if (n > 0) issue(0);
-        if (n > 1) issue(1);
-      }
-      c64 acc[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) acc[k] = czero<float>();
-      const int y = grp, kx = grp;
-      for (int c = 0; c < n; ++c) {
-        const uint32_t b = uint32_t(c & 1);
-        const bool ok = mbar_wait(bar + 8u * b, uint32_t(c >> 1) & 1u, TIMEOUT_NS);
-        if (!__syncthreads_and(ok)) {
-          if (tid == 0) atomicOr(err, 16);
-          return;
-        }
-        c64 v[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = *reinterpret_cast<const c64*>(sm + b * TILE_BYTES + sw_off(kx, t + 8 * q));
-        __syncthreads();  // the buffer is consumed: it becomes the group-transpose area
-        c64* gs = reinterpret_cast<c64*>(sm + b * TILE_BYTES) + grp * 64;
-        fft64_tma(v, t, gs, gpar, tw, true);  // inverse along y: lane t holds y = t + 8k
-#pragma unroll
-        for (int k = 0; k < 8; ++k) P[pidx(t + 8 * k, kx)] = v[k];
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = P[pidx(y, t + 8 * q)];
-        fft64_tma(v, t, gs, gpar, tw, true);  // inverse along x: lane t holds x = t + 8k
-        const Contrib cc = L.cd[s_list[c]];
-        const float f = float(occ[cc.occ]);
-        const c64* pp = src + size_t(cc.partner) * ng + size_t(z) * G * G + y * G;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          c64 a = v[k];
-          if (cc.conj) a.im = -a.im;
-          acc[k] = acc[k] + cmul(pp[t + 8 * k], a) * f;
-        }
-        __syncthreads();  // the buffer (transpose area) and P are free for the next contribution
-        if (tid == 0 && c + 2 < n) issue(c + 2);
-      }
-      c64* o = out + size_t(td.t) * ng + size_t(z) * G * G + y * G;
+      for (int q = 0; q < 8; ++q) v[q] = P[pidx(y, t + 8 * q)];
+      fft64_tma(v, t, gs, gpar, tw, true);  // inverse along x: lane t holds x = t + 8k
+      const Contrib cc = L.cd[s_list[c]];
+      const float f = float(occ[cc.occ]);
+      const c64* pp = src + size_t(cc.partner) * ng + size_t(z) * G * G + y * G;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        const int e = t + 8 * k;
-        o[e] = td.first ? czero<float>() - acc[k] : o[e] - acc[k];
+        c64 a = v[k];
+        if (cc.conj) a.im = -a.im;
+        acc[k] = acc[k] + cmul(pp[t + 8 * k], a) * f;
       }
-      return;
+      __syncthreads();  // the buffer (transpose area) and P are free for the next contribution
+      if (tid == 0 && c + 2 < n) issue(c + 2);
     }
-    bid -= L.nD;
+    c64* o = out + size_t(td.t) * ng + size_t(z) * G * G + y * G;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int e = t + 8 * k;
+      o[e] = td.first ? czero<float>() - acc[k] : o[e] - acc[k];
+    }
+    return;
   }
+  bid -= L.nD;
 
   if (bid < L.nA) {
     // ---------------- pass A ----------------
@@ -241,115 +234,6 @@ __global__ void __launch_bounds__(THREADS, 2)
     if (tid == 0 && !skip) tma_store_wait_all();
     return;
   }
-  bid -= L.nB;
-  if constexpr (FUSED) return;
-  if (bid < L.nC) {
-    // ---------------- pass C (two planes per CTA: z and z + G/2) ----------------
-    // The second plane loads into the B tile, unused by this role, while the first is transformed.
-    constexpr int H = G / 2;
-    const int z0 = bid % H, p = bid / H;
-    const PairDesc pd = L.pc[p];
-    const int orb = L.slotC * L.max_pairs + p;
-    if (tid == 0) {
-      mbar_arrive_expect_tx(bar, TILE_BYTES);
-      tma_load_5d(base + OFF_A, &tm_plane, 0, 0, z0, orb, 0, bar);
-      mbar_arrive_expect_tx(bar + 8, TILE_BYTES);
-      tma_load_5d(base + OFF_B, &tm_plane, 0, 0, z0 + H, orb, 0, bar + 8);
-    }
-    const bool skip = pair_skipped(pd, occ);
-    const int kx = grp;
-    c64* gs = reinterpret_cast<c64*>(sm + OFF_A) + grp * 64;
-    for (int h = 0; h < 2; ++h) {
-      const int z = z0 + h * H;
-      if (!mbar_wait(bar + 8u * h, 0, TIMEOUT_NS)) {
-        atomicOr(err, 4);
-        return;
-      }
-      if (skip) continue;  // uniform over the CTA; both loads still land before it exits
-      c64 v[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        v[q] = *reinterpret_cast<const c64*>(sm + (h ? OFF_B : OFF_A) + sw_off(kx, t + 8 * q));
-      // first plane: tile A consumed before it becomes the group-transpose area; second plane:
-      // every warp is done with the first plane's transpose areas
-      __syncthreads();
-      fft64_tma(v, t, gs, gpar, tw, true);  // inverse along y: lane t holds y = t + 8k
-#pragma unroll
-      for (int k = 0; k < 8; ++k) P[pidx(t + 8 * k, kx)] = v[k];
-      __syncthreads();
-      const int y = grp;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = P[pidx(y, t + 8 * q)];
-      fft64_tma(v, t, gs, gpar, tw, true);  // inverse along x: lane t holds x = t + 8k
-      c64* o = scratch + size_t(orb) * ng + size_t(z) * G * G + y * G;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) o[t + 8 * k] = v[k];
-    }
-    return;
-  }
-  bid -= L.nC;
-  {
-    // ---------------- pass D (half a plane per CTA) ----------------
-    // plane-major order: all targets of the batch at one z run together, so the two targets of a
-    // symmetric pair read its v_ij plane close in time (the second read hits L2), as do the
-    // partner planes shared by a tile row.  The v_ij and partner half-planes (16 KB each, one
-    // contiguous range apiece) stream through a ring of DS shared-memory slots by bulk copies,
-    // DS contributions ahead of the arithmetic, so the loads overlap without holding registers.
-    const int nt = L.nD / (2 * G);
-    const int z = (bid >> 1) / nt, half = bid & 1;
-    const TargetDesc td = L.td[(bid >> 1) % nt];
-    constexpr int EPT = G * G / (2 * THREADS);
-    constexpr uint32_t HB = G * G / 2 * sizeof(c64);  // bytes of a half plane
-    constexpr int DS = 3;                             // 3 x 32 KB below the twiddle table
-    const int e0 = half * (G * G / 2) + tid;
-    const size_t zoff = size_t(z) * G * G;
-    const size_t hoff = zoff + size_t(half) * (G * G / 2);
-    const int nc = td.cend - td.cbeg;
-    auto issue = [&](int i) {  // one thread
-      const Contrib cc = L.cd[td.cbeg + i - L.d_cbeg];
-      const int sl = i % DS;
-      const uint32_t dst = base + uint32_t(sl) * 2u * HB;
-      fence_proxy_async_smem();  // the slot's previous contents were read through the generic proxy
-      mbar_arrive_expect_tx(bar + 8u * sl, 2u * HB);
-      bulk_load(dst, scratch + (size_t(L.slotD) * L.max_pairs + cc.slot) * ng + hoff, HB, bar + 8u * sl);
-      bulk_load(dst + HB, src + size_t(cc.partner) * ng + hoff, HB, bar + 8u * sl);
-    };
-    if (tid == 0)
-      for (int i = 0; i < min(DS, nc); ++i) issue(i);
-    c64 acc[EPT];
-#pragma unroll
-    for (int u = 0; u < EPT; ++u) acc[u] = czero<float>();
-    for (int i = 0; i < nc; ++i) {
-      const int sl = i % DS;
-      const Contrib cc = L.cd[td.cbeg + i - L.d_cbeg];
-      const float f = float(occ[cc.occ]);
-      const bool ok = mbar_wait(bar + 8u * sl, (i / DS) & 1, TIMEOUT_NS);
-      // a skipped pair (d = 0) left its scratch slot unwritten: never multiply stale data by 0
-      if (ok && f != 0.f) {
-        const c64* sv = reinterpret_cast<const c64*>(sm + sl * 2 * HB);
-        const c64* sq = sv + G * G / 2;
-#pragma unroll
-        for (int u = 0; u < EPT; ++u) {
-          c64 a = sv[tid + u * THREADS];
-          if (cc.conj) a.im = -a.im;
-          acc[u] = acc[u] + cmul(sq[tid + u * THREADS], a) * f;
-        }
-      }
-      // every thread is done with slot sl before it is refilled; an expired wait ends the CTA
-      // uniformly
-      if (!__syncthreads_and(ok)) {
-        if (tid == 0) atomicOr(err, 8);
-        return;
-      }
-      if (tid == 0 && i + DS < nc) issue(i + DS);
-    }
-    c64* o = out + size_t(td.t) * ng + zoff + e0;
-#pragma unroll
-    for (int u = 0; u < EPT; ++u) {
-      const int e = u * THREADS;
-      o[e] = td.first ? czero<float>() - acc[u] : o[e] - acc[u];
-    }
-  }
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -412,20 +296,17 @@ void encode_tmap_4d_u64(CUtensorMap* map, const void* base, const uint64_t dims[
 }
 
 void exchange64_tma(pt_ctx* ctx, const ScheduleImpl& sch, const c64* src, const double* occ, const c64* tgt, int M,
-                    c64* out, const float* ktab, const c64* tw, cudaStream_t st, bool fused) {
+                    c64* out, const float* ktab, cudaStream_t st) {
   if (sch.B > MAXB) fail(PT_INVALID_ARG, "64^3 exchange schedule tile exceeds the parameter-block capacity");
   constexpr size_t ng = size_t(G) * G * G;
   const int maxp = sch.max_pairs;
-  const int ns = fused ? 3 : 4;  // scratch slots: one per role that holds pair fields
+  constexpr int ns = 3;  // scratch slots: one per role
   c64* scratch = static_cast<c64*>(ctx->get(ctx->tagged("exchange64_scratch"), size_t(ns) * maxp * ng * sizeof(c64)));
   int* err = static_cast<int*>(ctx->get("exchange_err", sizeof(int)));
   if (!ctx->defer_checks) PT_CUDA_CHECK(cudaMemsetAsync(err, 0, sizeof(int), st));  // else zeroed once per batch
   static DeviceOnce once;  // kernel attribute and the constant twiddle table are per device
   once([] {
-    PT_CUDA_CHECK(
-        cudaFuncSetAttribute(k_exchange64_tma<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    PT_CUDA_CHECK(
-        cudaFuncSetAttribute(k_exchange64_tma<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    PT_CUDA_CHECK(cudaFuncSetAttribute(k_exchange64_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     c64 h[G];
     for (int i = 0; i < G; ++i) {
       const double ang = -2.0 * M_PI * double(i) / double(G);
@@ -433,7 +314,6 @@ void exchange64_tma(pt_ctx* ctx, const ScheduleImpl& sch, const c64* src, const 
     }
     PT_CUDA_CHECK(cudaMemcpyToSymbol(c_tw64, h, sizeof(h)));
   });
-  (void)tw;
   // 5-D views (x mod 16, y, z, field, x / 16) of the [field][z][y][x] complex64 arrays: one copy
   // moves a whole 64 x 64 plane or slab as four 16-column sub-tiles of 128-byte rows (the x / 16
   // dimension, stride 128 B, outermost in the box), the shared-memory layout the line transforms read
@@ -455,8 +335,7 @@ void exchange64_tma(pt_ctx* ctx, const ScheduleImpl& sch, const c64* src, const 
     return np;
   };
   Launch L;
-  // launch k: A of batch k, B of batch k - 1, then C of k - 2 and D of k - 3 (four slots), or the
-  // fused CD of batch k - 2 (three slots); the roles of one launch always use distinct slots
+  // launch k: A of batch k, B of batch k - 1 and CD of batch k - 2, on distinct slots
   for (int k = 0; k < nb + ns - 1; ++k) {
     std::memset(&L, 0, sizeof(L));
     L.max_pairs = maxp;
@@ -464,14 +343,10 @@ void exchange64_tma(pt_ctx* ctx, const ScheduleImpl& sch, const c64* src, const 
       L.nA = G * copy_pairs(L.pa, k);
       L.slotA = k % ns;
     }
-    const int b = k - 1, c = k - 2, d = fused ? k - 2 : k - 3;
+    const int b = k - 1, d = k - 2;
     if (b >= 0 && b < nb) {
       L.nB = (G / 2) * copy_pairs(L.pb, b);
       L.slotB = b % ns;
-    }
-    if (!fused && c >= 0 && c < nb) {
-      L.nC = (G / 2) * copy_pairs(L.pc, c);
-      L.slotC = c % ns;
     }
     if (d >= 0 && d < nb) {
       const int t0 = sch.tgt_off[d], nt = sch.tgt_off[d + 1] - t0;
@@ -483,17 +358,13 @@ void exchange64_tma(pt_ctx* ctx, const ScheduleImpl& sch, const c64* src, const 
         if (sch.h_tgts[t0 + q].cend - sch.h_tgts[t0 + q].cbeg > 2 * MAXB)
           fail(PT_INVALID_ARG, "exchange batch: a target has more contributions than a tile allows");
       std::copy(sch.h_contribs.begin() + L.d_cbeg, sch.h_contribs.begin() + cend, L.cd);
-      L.nD = (fused ? G : 2 * G) * nt;
+      L.nD = G * nt;
       L.slotD = d % ns;
     }
-    const int grid = L.nA + L.nB + L.nC + L.nD;
+    const int grid = L.nA + L.nB + L.nD;
     if (grid == 0) continue;
-    if (fused)
-      PT_LAUNCH(k_exchange64_tma<true>, grid, THREADS, SMEM_BYTES, st, tm_src, tm_tgt, tm_plane, tm_slab, L, src, occ,
-                ktab, scratch, out, err);
-    else
-      PT_LAUNCH(k_exchange64_tma<false>, grid, THREADS, SMEM_BYTES, st, tm_src, tm_tgt, tm_plane, tm_slab, L, src,
-                occ, ktab, scratch, out, err);
+    PT_LAUNCH(k_exchange64_tma, grid, THREADS, SMEM_BYTES, st, tm_src, tm_tgt, tm_plane, tm_slab, L, src, occ, ktab,
+              scratch, out, err);
   }
 }
 

@@ -1,7 +1,4 @@
-// Compile-time pair-FFT exchange kernels (Sec. IV-A1, Eq. vxdiag) on cubic grids with side N, with
-// FT threads per CTA in the three tile kernels; included by the translation units that instantiate
-// them (exchange_fixed.cu: FT = 256; exchange_fixed_ft.cu: the other CTA sizes the batched form's
-// autotuner chooses from).
+// Compile-time pair-FFT exchange kernels (Sec. IV-A1, Eq. vxdiag) on cubic grids with side N.
 //
 // Four passes per pair batch, all on L2-resident pair fields (one scratch field per pair):
 //   plane:      rho = conj(src_i) tgt_j on one z-plane, FFT along x and y;
@@ -22,6 +19,7 @@ namespace pt {
 
 namespace {
 
+constexpr int FT = 256;  // threads per CTA of the tile kernels
 constexpr int AT = 256;  // threads per CTA of the accumulate kernel
 constexpr int AE = 4;    // elements per thread of the accumulate kernel
 
@@ -30,7 +28,7 @@ constexpr size_t tile_smem() {
   return size_t(N) * kPitch<N> * sizeof(cx<T>) + size_t(N) * sizeof(cx<T>);
 }
 
-template <int N, class T, int FT>
+template <int N, class T>
 __global__ void __launch_bounds__(FT) k_fx_fwd_plane(const cx<T>* __restrict__ src, const cx<T>* __restrict__ tgt,
                                                      const double* __restrict__ occ,
                                                      const PairDesc* __restrict__ pairs, cx<T>* __restrict__ scratch,
@@ -62,7 +60,7 @@ __global__ void __launch_bounds__(FT) k_fx_fwd_plane(const cx<T>* __restrict__ s
   }
 }
 
-template <int N, class T, int FT>
+template <int N, class T>
 __global__ void __launch_bounds__(FT) k_fx_column(cx<T>* __restrict__ scratch, const T* __restrict__ ktab,
                                                   const double* __restrict__ occ, const PairDesc* __restrict__ pairs,
                                                   const cx<T>* __restrict__ twg) {
@@ -97,7 +95,7 @@ __global__ void __launch_bounds__(FT) k_fx_column(cx<T>* __restrict__ scratch, c
   }
 }
 
-template <int N, class T, int FT>
+template <int N, class T>
 __global__ void __launch_bounds__(FT) k_fx_inv_plane(cx<T>* __restrict__ scratch, const double* __restrict__ occ,
                                                      const PairDesc* __restrict__ pairs,
                                                      const cx<T>* __restrict__ twg) {
@@ -162,30 +160,30 @@ __global__ void __launch_bounds__(AT) k_fx_accumulate(const cx<T>* __restrict__ 
   }
 }
 
-template <int N, class T, int FT>
+template <int N, class T>
 void set_fx_attrs() {
   static DeviceOnce once;
   once([] {
     const int bytes = int(tile_smem<N, T>());
     PT_CUDA_CHECK(
-        cudaFuncSetAttribute(k_fx_fwd_plane<N, T, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    PT_CUDA_CHECK(cudaFuncSetAttribute(k_fx_column<N, T, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+        cudaFuncSetAttribute(k_fx_fwd_plane<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    PT_CUDA_CHECK(cudaFuncSetAttribute(k_fx_column<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     PT_CUDA_CHECK(
-        cudaFuncSetAttribute(k_fx_inv_plane<N, T, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+        cudaFuncSetAttribute(k_fx_inv_plane<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
   });
 }
 
-// the four passes of one pair batch with FT threads per CTA in the three tile kernels
-template <int N, class T, int FT>
+// the four passes of one pair batch
+template <int N, class T>
 void batch_n(const cx<T>* src, const cx<T>* tgt, const double* occ, const PairDesc* pairs, int np,
              const TargetDesc* tgts, int nt, const Contrib* contribs, const T* ktab, const cx<T>* tw, cx<T>* scratch,
              cx<T>* out, cudaStream_t st) {
-  set_fx_attrs<N, T, FT>();
+  set_fx_attrs<N, T>();
   const size_t smem = tile_smem<N, T>();
   constexpr size_t NG = size_t(N) * N * N;
-  PT_LAUNCH((k_fx_fwd_plane<N, T, FT>), dim3(N, np), FT, smem, st, src, tgt, occ, pairs, scratch, tw);
-  PT_LAUNCH((k_fx_column<N, T, FT>), dim3(N, np), FT, smem, st, scratch, ktab, occ, pairs, tw);
-  PT_LAUNCH((k_fx_inv_plane<N, T, FT>), dim3(N, np), FT, smem, st, scratch, occ, pairs, tw);
+  PT_LAUNCH((k_fx_fwd_plane<N, T>), dim3(N, np), FT, smem, st, src, tgt, occ, pairs, scratch, tw);
+  PT_LAUNCH((k_fx_column<N, T>), dim3(N, np), FT, smem, st, scratch, ktab, occ, pairs, tw);
+  PT_LAUNCH((k_fx_inv_plane<N, T>), dim3(N, np), FT, smem, st, scratch, occ, pairs, tw);
   const unsigned chunks = unsigned((NG + AT * AE - 1) / (AT * AE));
   PT_LAUNCH(k_fx_accumulate<T>, dim3(chunks, nt), AT, 0, st, scratch, src, occ, tgts, contribs, out, NG);
 }

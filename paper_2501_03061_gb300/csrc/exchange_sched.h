@@ -44,18 +44,21 @@ void exchange_batch_generic(const GridPlan& gp, const cx<T>* src, const cx<T>* t
                             const PairDesc* pairs, int np, const TargetDesc* tgts, int nt, const Contrib* contribs,
                             const T* ktab, const cx<T>* tw, cx<T>* scratch, cx<T>* out, cudaStream_t st);
 // the same passes with compile-time FFT kernels for a cubic grid of side n (fixed_cubic)
-// (ft: threads per CTA of the tile kernels, 256, or in FP32 also 128 or 512)
 template <class T>
 void exchange_batch_fixed(int n, const cx<T>* src, const cx<T>* tgt, const double* occ, const PairDesc* pairs, int np,
                           const TargetDesc* tgts, int nt, const Contrib* contribs, const T* ktab, const cx<T>* tw,
-                          cx<T>* scratch, cx<T>* out, cudaStream_t st, int ft = 256);
+                          cx<T>* scratch, cx<T>* out, cudaStream_t st);
 double kernel_value(const pt_kernel& k, double G2);
 
 bool exchange64_applies(const pt_grid& g);
-// FP32 64^3 path with TMA staging; sets a device error word on a wait timeout (see exchange_check)
-// fused: the three-role form (A, B, and CD: C's inverse plane transforms inside the accumulate)
+// FP32 exchange on cubic grids with whole lines in registers (exchange_lines.cu); budget: bytes of pair fields per
+// tile; returns the pair FFTs
+bool exchange_lines_applies(const pt_ctx* ctx, const pt_grid& g);
+long long exchange_lines(pt_ctx* ctx, const c64* src, const double* occ, int N, const c64* tgt, int M, bool sym, c64* out,
+                         const pt_grid& g, const pt_kernel& k, size_t budget, cudaStream_t st);
+// FP32 64^3 path with TMA staging (engine 3); sets a device error word on a wait timeout (see exchange_check)
 void exchange64_tma(pt_ctx* ctx, const ScheduleImpl& sch, const c64* src, const double* occ, const c64* tgt, int M,
-                    c64* out, const float* ktab, const c64* tw, cudaStream_t st, bool fused = false);
+                    c64* out, const float* ktab, cudaStream_t st);
 // FP32 64^3 path as one persistent cooperative launch (exchange64_persist.cu); returns the pair FFTs
 long long exchange64_persist(pt_ctx* ctx, const c64* src, const double* occ, int N, const c64* tgt, int M, bool sym,
                              c64* out, const float* ktab, const c64* tw, cudaStream_t st);

@@ -12,6 +12,8 @@ struct Term {
 };
 
 // ---- exchange (exchange.cu) ----
+// the FP32 line kernels apply (exchange_lines.cu)
+bool exchange_lines_applies(const pt_ctx* ctx, const pt_grid& g);
 // largest pair-tile side of the 64^3 TMA pipeline (its batch descriptors travel in the kernel
 // parameters: 16 bytes x (5 B^2 + 2 B) of the 32 KB parameter space)
 constexpr int kExchange64MaxTile = 16;
