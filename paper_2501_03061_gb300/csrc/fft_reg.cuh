@@ -227,7 +227,7 @@ __device__ __forceinline__ void short_dft(cx<T>* a) {
 
 // the split of a line length: the shorter factor first, coprime where the length allows it
 constexpr int first_factor(int n) {
-  return n == 16 ? 4 : n == 20 ? 4 : n == 24 ? 3 : n == 30 ? 5 : n == 32 ? 4 : n == 36 ? 4 : n == 40 ? 5
+  return n == 18 ? 2 : n == 25 ? 5 : n == 27 ? 3 : n == 45 ? 5 : n == 50 ? 5 : n == 16 ? 4 : n == 20 ? 4 : n == 24 ? 3 : n == 30 ? 5 : n == 32 ? 4 : n == 36 ? 4 : n == 40 ? 5
          : n == 48 ? 3 : n == 54 ? 6 : n == 60 ? 5 : n == 64 ? 8 : 0;
 }
 

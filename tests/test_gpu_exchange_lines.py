@@ -59,6 +59,30 @@ def test_lines_match_oracle(ctx, n, N, M, tile):
     assert np.linalg.norm(out - ref) <= TOL * np.linalg.norm(ref)
 
 
+LENGTHS = [16, 18, 20, 24, 25, 27, 30, 32, 36, 40, 45, 48, 50, 54, 60, 64]
+
+
+@pytest.mark.parametrize("k", range(len(LENGTHS)))
+@pytest.mark.parametrize("N,M,tile", [(4, 0, 3), (3, 5, 8)])
+def test_axes_match_oracle(ctx, k, N, M, tile):
+    """Grids that are not cubic: every length on every axis, odd products among them."""
+    from oracle import ptim_oracle as O
+    from paper_2501_03061_gb300 import synth
+    rng = np.random.default_rng(900 + k)
+    nx, ny, nz = LENGTHS[k], LENGTHS[(k + 5) % 16], LENGTHS[(k + 11) % 16]
+    cell = synth.Cell((nx, ny, nz), (0.3 * nx, 0.34 * ny, 0.32 * nz))
+    src = rng.standard_normal((N, nz, ny, nx)) + 1j * rng.standard_normal((N, nz, ny, nx))
+    tgt = rng.standard_normal((M, nz, ny, nx)) + 1j * rng.standard_normal((M, nz, ny, nx)) if M else None
+    src = src.astype(np.complex64).astype(np.complex128)
+    tgt = tgt.astype(np.complex64).astype(np.complex128) if M else None
+    occ = np.linspace(1.0, 0.0, N)
+    kernel = {"type": 1, "mu": synth.SCREENED_MU}
+    K = O.exchange_kernel(O.grid_of(cell), 1, synth.SCREENED_MU)
+    ref = O.apply_exchange(src, occ, src if tgt is None else tgt, K)
+    out = run(ctx, cell, src, occ, tgt, tile, kernel)
+    assert np.linalg.norm(out - ref) <= TOL * np.linalg.norm(ref)
+
+
 @pytest.mark.parametrize("n,N", [(16, 70), (24, 40), (36, 30), (48, 18), (60, 14)])
 def test_one_group_per_column(ctx, n, N):
     """Enough targets that the last pass runs one group of threads per column; the tile kernels
