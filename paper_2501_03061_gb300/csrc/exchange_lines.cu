@@ -141,12 +141,13 @@ long long exchange_lines(pt_ctx* ctx, const c64* src, const double* occ, int N, 
   std::swap(gt.nx, gt.ny);
   std::swap(gt.L[0], gt.L[1]);
   const float* kt = static_cast<const float*>(kernel_table(ctx, gt, k, PT_FP32));
-  c64* scratch = static_cast<c64*>(
-      ctx->get(ctx->tagged("exchange_scratch"), size_t(std::min(B, N)) * size_t(std::min(B, M)) * field));
+  // as few tiles as the side allows, all of about the same size (36^3 N = 75: 25 + 25 + 25 instead of 37 + 37 + 1)
   const int nb = (N + B - 1) / B, mb = (M + B - 1) / B;
-  for (int J = 0; J < mb; ++J)
-    for (int I = 0; I < (sym ? J + 1 : nb); ++I) {
-      const Tile t{I * B, std::min(B, N - I * B), J * B, std::min(B, M - J * B), int(sym), int(sym && I == J), int(I == 0)};
+  const int bi = (N + nb - 1) / nb, bj = (M + mb - 1) / mb;
+  c64* scratch = static_cast<c64*>(ctx->get(ctx->tagged("exchange_scratch"), size_t(bi) * bj * field));
+  for (int J = 0; J * bj < M; ++J)
+    for (int I = 0; sym ? I <= J : I * bi < N; ++I) {
+      const Tile t{I * bi, std::min(bi, N - I * bi), J * bj, std::min(bj, M - J * bj), int(sym), int(sym && I == J), int(I == 0)};
       if (!fixed_cubic(g)) {
         exchange_tile_axes(g, t, src, tgt, occ, kt, scratch, out, ctx->num_sms, st);
         continue;
