@@ -9,6 +9,8 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "packed.cuh"
+#include "split_sum.cuh"
 
 namespace pt {
 
@@ -99,36 +101,57 @@ __global__ void __launch_bounds__(GTHREADS) k_gram(const cx<T>* __restrict__ A, 
     }
 }
 
+// asynchronous 8-byte copy global -> shared (zeros where !valid; src must be a readable address all the same)
+__device__ __forceinline__ void copy8(c64* dst, const c64* src, bool valid) {
+  const unsigned d = unsigned(__cvta_generic_to_shared(dst));
+  const int bytes = valid ? 8 : 0;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(bytes));
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N));
+}
+
 // FP32 Gram tile of 64 x 64 outputs, 4 x 4 complex per thread, 16 grid points per stage; the
 // per-stage sums are folded into Kahan-compensated totals.  With herm, only tiles on or above
-// the diagonal run (the reduction mirrors the rest).
+// the diagonal run (the reduction mirrors the rest).  Bound by FP32 arithmetic and its issue: the next
+// stage's operands arrive by asynchronous copies while this one is multiplied, and a complex product is
+// two packed instructions.
 constexpr int G4T = 64, G4K = 16, G4THREADS = 256;
 
 __global__ void __launch_bounds__(G4THREADS, 2) k_gram64(const c64* __restrict__ A, const c64* __restrict__ B,
                                                          int N1, int N2, size_t ng, size_t chunk, int herm,
                                                          c128* __restrict__ part) {
   if (herm && blockIdx.y < blockIdx.x) return;
-  __shared__ c64 As[G4K][G4T + 1];
-  __shared__ c64 Bs[G4K][G4T + 1];
+  __shared__ c64 As[2][G4K][G4T + 1];
+  __shared__ c64 Bs[2][G4K][G4T + 1];
   const int i0 = blockIdx.x * G4T, j0 = blockIdx.y * G4T;
   const size_t r_begin = size_t(blockIdx.z) * chunk;
   const size_t r_end = std::min(ng, r_begin + chunk);
   const int tid = threadIdx.x;
   const int ti = tid % 16, tj = tid / 16;
-  Acc<float> sre[4][4], sim[4][4];
-  for (size_t r0 = r_begin; r0 < r_end; r0 += G4K) {
+  auto fetch = [&](size_t r0, int buf) {
 #pragma unroll
     for (int pass = 0; pass < (G4T * G4K) / G4THREADS; ++pass) {
       const int e = tid + pass * G4THREADS;
       const int k = e % G4K, o = e / G4K;
       const size_t r = r0 + k;
-      c64 va = czero<float>(), vb = czero<float>();
-      if (r < r_end) {
-        if (i0 + o < N1) va = A[size_t(i0 + o) * ng + r];
-        if (j0 + o < N2) vb = B[size_t(j0 + o) * ng + r];
-      }
-      As[k][o] = va;
-      Bs[k][o] = vb;
+      const bool va = r < r_end && i0 + o < N1, vb = r < r_end && j0 + o < N2;
+      copy8(&As[buf][k][o], va ? A + size_t(i0 + o) * ng + r : A, va);
+      copy8(&Bs[buf][k][o], vb ? B + size_t(j0 + o) * ng + r : B, vb);
+    }
+    copy_commit();
+  };
+  Acc<float> sre[4][4], sim[4][4];
+  int buf = 0;
+  if (r_begin < r_end) fetch(r_begin, 0);
+  for (size_t r0 = r_begin; r0 < r_end; r0 += G4K, buf ^= 1) {
+    if (r0 + G4K < r_end) {
+      fetch(r0 + G4K, buf ^ 1);
+      copy_wait<1>();
+    } else {
+      copy_wait<0>();
     }
     __syncthreads();
     c64 acc[4][4];
@@ -138,15 +161,15 @@ __global__ void __launch_bounds__(G4THREADS, 2) k_gram64(const c64* __restrict__
       for (int b = 0; b < 4; ++b) acc[a][b] = czero<float>();
 #pragma unroll 4
     for (int k = 0; k < G4K; ++k) {
-      c64 av[4], bv[4];
+      c64 av[4];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = conjc(As[k][ti + 16 * a]);
+      for (int a = 0; a < 4; ++a) av[a] = As[buf][k][ti + 16 * a];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) bv[b] = Bs[k][tj + 16 * b];
+      for (int b = 0; b < 4; ++b) {
+        const c64 bv = Bs[buf][k][tj + 16 * b], bx = c64{bv.im, -bv.re};  // conj(a) b = Re(a) b + Im(a) (-i b)
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) cfma(acc[a][b], av[a], bv[b]);
+        for (int a = 0; a < 4; ++a) acc[a][b] = rl::pfma(bx, av[a].im, rl::pfma(bv, av[a].re, acc[a][b]));
+      }
     }
 #pragma unroll
     for (int a = 0; a < 4; ++a)
@@ -155,7 +178,7 @@ __global__ void __launch_bounds__(G4THREADS, 2) k_gram64(const c64* __restrict__
         sre[a][b].add(acc[a][b].re);
         sim[a][b].add(acc[a][b].im);
       }
-    __syncthreads();
+    __syncthreads();  // this buffer is refilled in the next round
   }
   c128* P = part + size_t(blockIdx.z) * N1 * N2;
 #pragma unroll
@@ -169,20 +192,16 @@ __global__ void __launch_bounds__(G4THREADS, 2) k_gram64(const c64* __restrict__
 
 // C = scale * sum of split partials; herm_tile > 0: elements whose tile row is below the tile
 // column were not computed and are taken as the conjugate of the mirrored element
-__global__ void k_reduce_parts(const c128* __restrict__ part, int nsplit, int N1, int N2, double scale,
-                               int herm_tile, c128* __restrict__ C) {
-  const size_t n = size_t(N1) * N2;
-  const size_t e = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= n) return;
+template <int G>
+__global__ void __launch_bounds__(SUM_THREADS) k_reduce_parts(const c128* __restrict__ part, int nsplit, int N1, int N2,
+                                                              double scale, int herm_tile, c128* __restrict__ C) {
+  const size_t n = size_t(N1) * N2, e = split_entry<G>();
   const int i = int(e / N2), j = int(e % N2);
   const bool mirror = herm_tile > 0 && (i / herm_tile) > (j / herm_tile);
   const size_t src = mirror ? size_t(j) * N2 + i : e;
-  double re = 0, im = 0;
-  for (int s = 0; s < nsplit; ++s) {
-    re += part[size_t(s) * n + src].re;
-    im += part[size_t(s) * n + src].im;
-  }
-  C[e] = mirror ? c128{re * scale, -im * scale} : c128{re * scale, im * scale};
+  double re, im;
+  if (split_sum<G>(nsplit, e < n, [&](int s) { return part[size_t(s) * n + src]; }, re, im))
+    C[e] = mirror ? c128{re * scale, -im * scale} : c128{re * scale, im * scale};
 }
 
 // ---------------------------------------------------------------- rotate (A Bm + E) ----
@@ -253,6 +272,89 @@ __global__ void __launch_bounds__(RTHREADS) k_rotate(const cx<T>* __restrict__ A
       if (r >= ng) continue;
       const size_t idx = size_t(j) * ng + r;
       cx<T> v = cmul(alpha, acc[a][b]);
+#pragma unroll
+      for (int t = 0; t < 3; ++t)
+        if (epi.e[t]) v = v + cmul(epi.c[t], epi.e[t][idx]);
+      out[idx] = v;
+    }
+  }
+}
+
+// FP32 B operand of a rotation, converted once: an FP64 instruction issues every 64 cycles on this part, and
+// every point tile of k_rotate would convert all of B again
+__global__ void __launch_bounds__(256) k_rot_b32(const c128* __restrict__ B, int ldb, int N1, int N2, c64* __restrict__ out) {
+  const int e = blockIdx.x * 256 + threadIdx.x;
+  if (e >= N1 * N2) return;
+  const int k = e / N2, j = e - k * N2;
+  out[e] = to_cx<float>(B[size_t(k) * ldb + j]);
+}
+
+// The FP32 form of k_rotate: the same tile, the next stage's operands arriving by asynchronous copies, a complex
+// product in two packed instructions (in the order of cfma, so the results are the same bits)
+__global__ void __launch_bounds__(RTHREADS, 3) k_rotate32(const c64* __restrict__ A, const c64* __restrict__ Bm, int N1, int N2,
+                                                       size_t ng, c64 alpha, Epi<float> epi, c64* __restrict__ out) {
+  __shared__ c64 As[2][KC][RT];
+  __shared__ c64 Bs[2][KC][JT];
+  const size_t r0 = size_t(blockIdx.x) * RT;
+  const int j0 = blockIdx.y * JT;
+  const int tid = threadIdx.x;
+  const int tr = tid % 32, tj = tid / 32;  // 32 x 8
+  auto fetch = [&](int k0, int buf) {
+#pragma unroll
+    for (int pass = 0; pass < (KC * RT) / RTHREADS; ++pass) {
+      const int e = tid + pass * RTHREADS;
+      const int r = e % RT, kk = e / RT;
+      const bool v = k0 + kk < N1 && r0 + r < ng;
+      copy8(&As[buf][kk][r], v ? A + size_t(k0 + kk) * ng + r0 + r : A, v);
+    }
+#pragma unroll
+    for (int pass = 0; pass < (KC * JT) / RTHREADS; ++pass) {
+      const int e = tid + pass * RTHREADS;
+      const int j = e % JT, kk = e / JT;
+      const bool v = k0 + kk < N1 && j0 + j < N2;
+      copy8(&Bs[buf][kk][j], v ? Bm + size_t(k0 + kk) * N2 + j0 + j : Bm, v);
+    }
+    copy_commit();
+  };
+  c64 acc[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[a][b] = czero<float>();
+  int buf = 0;
+  fetch(0, 0);
+  for (int k0 = 0; k0 < N1; k0 += KC, buf ^= 1) {
+    if (k0 + KC < N1) {
+      fetch(k0 + KC, buf ^ 1);
+      copy_wait<1>();
+    } else {
+      copy_wait<0>();
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < KC; ++kk) {
+      c64 av[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) av[a] = As[buf][kk][tr + 32 * a];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const c64 bv = Bs[buf][kk][tj + 8 * b], bx = c64{-bv.im, bv.re};
+#pragma unroll
+        for (int a = 0; a < 4; ++a) acc[a][b] = rl::pfma(bx, av[a].im, rl::pfma(bv, av[a].re, acc[a][b]));
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const int j = j0 + tj + 8 * b;
+    if (j >= N2) continue;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const size_t r = r0 + tr + 32 * a;
+      if (r >= ng) continue;
+      const size_t idx = size_t(j) * ng + r;
+      c64 v = cmul(alpha, acc[a][b]);
 #pragma unroll
       for (int t = 0; t < 3; ++t)
         if (epi.e[t]) v = v + cmul(epi.c[t], epi.e[t][idx]);
@@ -345,9 +447,7 @@ void gram(pt_ctx* ctx, const cx<T>* A, const cx<T>* B, int N1, int N2, size_t ng
     herm = false;
     PT_LAUNCH(k_gram<T>, dim3(ti, tj, splits), GTHREADS, 0, st, A, B, N1, N2, ng, chunk, part);
   }
-  const size_t n = size_t(N1) * N2;
-  PT_LAUNCH(k_reduce_parts, dim3(unsigned((n + 255) / 256)), 256, 0, st, part, splits, N1, N2, scale,
-            herm ? tile : 0, C);
+  PT_LAUNCH_SPLIT_SUM(k_reduce_parts, size_t(N1) * N2, 1, splits, st, part, splits, N1, N2, scale, herm ? tile : 0, C);
 }
 
 template <class T>
@@ -383,7 +483,13 @@ void rotate(pt_ctx* ctx, const cx<T>* A, const c128* Bm, int ldb, int N1, int N2
     epi.c[t] = (t < nterms) ? to_cx<T>(terms[t].c) : czero<T>();
   }
   dim3 grid(unsigned((ng + RT - 1) / RT), unsigned((N2 + JT - 1) / JT));
-  PT_LAUNCH(k_rotate<T>, grid, RTHREADS, 0, st, A, Bm, ldb, N1, N2, ng, to_cx<T>(alpha), epi, out);
+  if constexpr (sizeof(T) == 4) {
+    c64* b32 = static_cast<c64*>(ctx->get("rot_b32", size_t(N1) * N2 * sizeof(c64)));
+    PT_LAUNCH(k_rot_b32, (N1 * N2 + 255) / 256, 256, 0, st, Bm, ldb, N1, N2, b32);
+    PT_LAUNCH(k_rotate32, grid, RTHREADS, 0, st, A, b32, N1, N2, ng, to_cx<T>(alpha), epi, out);
+  } else {
+    PT_LAUNCH(k_rotate<T>, grid, RTHREADS, 0, st, A, Bm, ldb, N1, N2, ng, to_cx<T>(alpha), epi, out);
+  }
 }
 
 template <class T>

@@ -25,6 +25,7 @@
 #include <cstring>
 
 #include "internal.h"
+#include "split_sum.cuh"
 #include "tma.cuh"
 
 namespace pt {
@@ -329,11 +330,12 @@ __global__ void __launch_bounds__(THREADS, 1)
 }
 
 // C[i][j] = scale * sum_split part[split][tile][row][col]; herm: mirror the tiles not computed
-__global__ void k_gram_tc_reduce(const double* __restrict__ part, int nsplit, int ntiles, int tiles_j, int N1, int N2,
-                                 double scale, int herm, c128* __restrict__ C) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= N1 * N2) return;
-  int i = e / N2, j = e % N2;
+template <int G>
+__global__ void __launch_bounds__(SUM_THREADS) k_gram_tc_reduce(const double* __restrict__ part, int nsplit, int ntiles,
+                                                                int tiles_j, int N1, int N2, double scale, int herm,
+                                                                c128* __restrict__ C) {
+  const size_t e = split_entry<G>();
+  int i = int(e / N2), j = int(e % N2);
   bool mirror = false;
   if (herm && (j / TN) < (i / TM)) {
     mirror = true;
@@ -343,13 +345,15 @@ __global__ void k_gram_tc_reduce(const double* __restrict__ part, int nsplit, in
   }
   const int tile = (i / TM) * tiles_j + (j / TN);
   const int r = i % TM, c = j % TN;
-  double re = 0, im = 0;
-  for (int s = 0; s < nsplit; ++s) {
-    const double* p = part + (size_t(s) * ntiles + tile) * 128 * TN;
-    re += p[size_t(r) * TN + c];
-    im += p[size_t(TM + r) * TN + c];
-  }
-  C[e] = mirror ? c128{re * scale, -im * scale} : c128{re * scale, im * scale};
+  double re, im;
+  const bool owner = split_sum<G>(
+      nsplit, e < size_t(N1) * N2,
+      [&](int s) {
+        const double* p = part + (size_t(s) * ntiles + tile) * 128 * TN;
+        return c128{p[size_t(r) * TN + c], p[size_t(TM + r) * TN + c]};
+      },
+      re, im);
+  if (owner) C[e] = mirror ? c128{re * scale, -im * scale} : c128{re * scale, im * scale};
 }
 
 }  // namespace
@@ -390,8 +394,8 @@ void gram_tc(pt_ctx* ctx, const c64* A, const c64* B, int N1, int N2, size_t ng,
   encode_tmap_4d_f32(&tb, B, db, sb, boxb, CU_TENSOR_MAP_SWIZZLE_128B);
   TileArgs P{N1, N2, tj, herm ? 1 : 0, stages_total, sps, split3 ? 1 : 0, std::max(1, ctx->tc_period)};
   PT_LAUNCH(k_gram_tc, dim3(ntiles, splits), THREADS, SMEM_BYTES, st, ta, tb, P, part, err);
-  PT_LAUNCH(k_gram_tc_reduce, (N1 * N2 + 255) / 256, 256, 0, st, part, splits, ntiles, tj, N1, N2, scale,
-            herm ? 1 : 0, C);
+  PT_LAUNCH_SPLIT_SUM(k_gram_tc_reduce, size_t(N1) * N2, 1, splits, st, part, splits, ntiles, tj, N1, N2, scale,
+                      herm ? 1 : 0, C);
 }
 
 void gram_tc_check(pt_ctx* ctx, cudaStream_t st) {

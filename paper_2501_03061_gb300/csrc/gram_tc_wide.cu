@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "split_sum.cuh"
 #include "tma.cuh"
 
 namespace pt {
@@ -333,17 +334,17 @@ __global__ void __launch_bounds__(W_THREADS, 1)
 // C_m[i][j] = scale * sum_split part[split][tile][row][col] through a block lookup: entry
 // (m, i / 64, j / 64) = tile * 4 + half * 2 + mirror (-1: not computed); a mirrored block is the
 // conjugate transpose of block (j / 64, i / 64)
-__global__ void k_gram_tc_wide_reduce(const double* __restrict__ part, int nsplit, int ntiles, const int* __restrict__ lut,
-                                      int nbi, int nbj, int N1, int N2, double scale, c128* __restrict__ C0,
-                                      c128* __restrict__ C1) {
-  const size_t n = size_t(N1) * N2;
-  const size_t e = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+template <int G>
+__global__ void __launch_bounds__(SUM_THREADS) k_gram_tc_wide_reduce(const double* __restrict__ part, int nsplit, int ntiles,
+                                                                     const int* __restrict__ lut, int nbi, int nbj, int N1,
+                                                                     int N2, double scale, c128* __restrict__ C0,
+                                                                     c128* __restrict__ C1) {
+  const size_t e = split_entry<G>();
   const int m = int(blockIdx.y);
-  if (e >= n) return;
+  const bool in = e < size_t(N1) * N2;
   c128* C = m == 0 ? C0 : C1;
   int i = int(e / N2), j = int(e % N2);
-  const int code = lut[(size_t(m) * nbi + i / WB) * nbj + j / WB];
-  if (code < 0) return;
+  const int code = in ? lut[(size_t(m) * nbi + i / WB) * nbj + j / WB] : -1;
   const int tile = code >> 2, half = (code >> 1) & 1, mirror = code & 1;
   if (mirror) {
     const int t = i;
@@ -351,13 +352,15 @@ __global__ void k_gram_tc_wide_reduce(const double* __restrict__ part, int nspli
     j = t;
   }
   const int r = i % WB, c = half * WB + j % WB;
-  double re = 0, im = 0;
-  for (int s = 0; s < nsplit; ++s) {
-    const double* p = part + (size_t(s) * ntiles + tile) * 128 * WN;
-    re += p[size_t(r) * WN + c];
-    im += p[size_t(WB + r) * WN + c];
-  }
-  C[e] = mirror ? c128{re * scale, -im * scale} : c128{re * scale, im * scale};
+  double re, im;
+  const bool owner = split_sum<G>(
+      nsplit, code >= 0,
+      [&](int s) {
+        const double* p = part + (size_t(s) * ntiles + tile) * 128 * WN;
+        return c128{p[size_t(r) * WN + c], p[size_t(WB + r) * WN + c]};
+      },
+      re, im);
+  if (owner) C[e] = mirror ? c128{re * scale, -im * scale} : c128{re * scale, im * scale};
 }
 
 struct WidePlan {
@@ -450,8 +453,8 @@ void gram_tc_wide(pt_ctx* ctx, const c64* A, const c64* B0, c128* C0, const c64*
             err);
   const size_t n = size_t(N1) * N2;
   const int nbi = (N1 + WB - 1) / WB, nbj = (N2 + WB - 1) / WB;
-  PT_LAUNCH(k_gram_tc_wide_reduce, dim3(unsigned((n + 255) / 256), two ? 2u : 1u), 256, 0, st, part, splits,
-            pl->ntiles, pl->lut, nbi, nbj, N1, N2, scale, C0, C1);
+  PT_LAUNCH_SPLIT_SUM(k_gram_tc_wide_reduce, n, two ? 2u : 1u, splits, st, part, splits, pl->ntiles, pl->lut, nbi, nbj, N1,
+                      N2, scale, C0, C1);
 }
 
 }  // namespace pt
