@@ -5,11 +5,13 @@
 //
 // Density: chi = Phi sigma (the library's rotation, tensor cores in the FP32 forms), then
 // rho(r) = spin * Re sum_j chi_j(r) conj(phi_j(r)) in one streaming pass over both blocks
-// (2 N Ng complex reads, HBM bound), products in the block's precision and sums in FP64.
-// Potential: one FP64 3-D FFT of rho through the generic tile kernels (x/y plane pass, z column
-// pass that applies 4 pi/|G|^2 / Ng and transforms back, inverse y/x plane pass), whose last pass
-// also evaluates the LDA point by point, adds V_loc and writes the total local potential, with
-// per-plane partial sums of the Hartree and xc energies.  All of it is Ng-sized work.
+// (2 N Ng complex reads, HBM bound), products in the block's precision, sums to 48 bits or more.
+// Potential: one FP64 3-D FFT of the real rho, axis by axis on the half spectrum kx <= nx/2: two real rows make
+// one complex x line, y and z lines run on nx/2 + 1 columns, the z pass applies 4 pi/|G|^2 / Ng and transforms
+// back, and the last x pass evaluates the LDA point by point, adds V_loc and writes the total local potential.
+// Small tiles (4 x lines, 8 columns) give every pass 2-4 CTAs per SM: FP64 issues at 1/64 rate, so a pass
+// on nz of the 152 SMs is bound by that many FP64 pipes.  60^3: 114 us against 303 us of whole-plane tiles on the
+// full spectrum, of which the LDA's transcendentals took 100.
 #include <algorithm>
 
 #include "fft.cuh"
@@ -19,8 +21,10 @@ namespace pt {
 
 namespace {
 
-constexpr int NT = 512;
-constexpr int MAXE = kMaxDim * kMaxDim;
+constexpr int NT = 64;    // threads per CTA of the FFT passes
+constexpr int XL = 4;     // x lines (pairs of rows) per CTA
+constexpr int CL = 8;     // columns per CTA of the y and z passes
+constexpr int CP = CL + 1;  // their pitch
 constexpr double kPi = 3.14159265358979323846;
 
 // Perdew-Zunger correlation of the unpolarised gas (rs >= 1: gamma/(1 + beta1 sqrt(rs) + beta2 rs);
@@ -31,18 +35,20 @@ __device__ __forceinline__ void lda_point(double rho, double& eps, double& v) {
     v = 0.0;
     return;
   }
-  const double ex = -0.75 * cbrt(3.0 * rho / kPi);
-  const double rs = cbrt(3.0 / (4.0 * kPi * rho));
+  // t = 1/rs: one cube root serves rs = t^{-1}, sqrt(rs) = t^{-1/2} and (3 rho/pi)^{1/3} = (9/(4 pi^2))^{1/3} t
+  constexpr double cx = 0.75 * 0.61088705770857191;  // 3/4 (9/(4 pi^2))^{1/3}
+  const double t = cbrt(4.0 * kPi / 3.0 * rho);
+  const double ex = -cx * t;
   double ec, vc;
-  if (rs >= 1.0) {
+  if (t <= 1.0) {
     const double gamma = -0.1423, b1 = 1.0529, b2 = 0.3334;
-    const double s = sqrt(rs);
-    const double den = 1.0 + b1 * s + b2 * rs;
-    ec = gamma / den;
-    vc = ec * (1.0 + (7.0 / 6.0) * b1 * s + (4.0 / 3.0) * b2 * rs) / den;
+    const double s = rsqrt(t), rs = s * s;
+    const double inv = 1.0 / (1.0 + b1 * s + b2 * rs);
+    ec = gamma * inv;
+    vc = ec * (1.0 + (7.0 / 6.0) * b1 * s + (4.0 / 3.0) * b2 * rs) * inv;
   } else {
     const double a = 0.0311, b = -0.048, c = 0.0020, d = -0.0116;
-    const double l = log(rs);
+    const double l = -log(t), rs = 1.0 / t;
     ec = a * l + b + c * rs * l + d * rs;
     vc = a * l + (b - a / 3.0) + (2.0 / 3.0) * c * rs * l + (2.0 * d - c) / 3.0 * rs;
   }
@@ -50,11 +56,29 @@ __device__ __forceinline__ void lda_point(double rho, double& eps, double& v) {
   v = (4.0 / 3.0) * ex + vc;
 }
 
+// running sum of n terms: in FP32 as an unevaluated pair (two-sum: each addition's rounding error is kept, so the
+// sum is good to ~n 2^-48), since an FP64 addition of a converted term costs 128 issue cycles on this part
+template <class T>
+struct RunSum {
+  T s = T(0), e = T(0);
+  __device__ __forceinline__ void add(T x) {
+    if constexpr (sizeof(T) == 8) {
+      s += x;
+    } else {
+      const T n = __fadd_rn(s, x), b = __fsub_rn(n, s);
+      e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(n, b)), __fsub_rn(x, b)));
+      s = n;
+    }
+  }
+  // an overflowed sum is itself (its error term is not a number)
+  __device__ __forceinline__ double value() const { return isfinite(s) ? double(s) + double(e) : double(s); }
+};
+
 template <class T>
 __global__ void __launch_bounds__(256) k_density(const cx<T>* __restrict__ chi, const cx<T>* __restrict__ phi, int N,
                                                  size_t ng, double spin, double* __restrict__ rho) {
   for (size_t r = size_t(blockIdx.x) * blockDim.x + threadIdx.x; r < ng; r += size_t(gridDim.x) * blockDim.x) {
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    RunSum<T> acc[4];
     int j = 0;
     for (; j + 4 <= N; j += 4) {
       cx<T> a[4], b[4];
@@ -64,99 +88,117 @@ __global__ void __launch_bounds__(256) k_density(const cx<T>* __restrict__ chi, 
         b[u] = phi[size_t(j + u) * ng + r];
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) acc[u] += double(a[u].re * b[u].re + a[u].im * b[u].im);
+      for (int u = 0; u < 4; ++u) acc[u].add(a[u].re * b[u].re + a[u].im * b[u].im);
     }
     for (; j < N; ++j) {
       const cx<T> a = chi[size_t(j) * ng + r], b = phi[size_t(j) * ng + r];
-      acc[0] += double(a.re * b.re + a.im * b.im);
+      acc[0].add(a.re * b.re + a.im * b.im);
     }
-    rho[r] = spin * ((acc[0] + acc[1]) + (acc[2] + acc[3]));
+    rho[r] = spin * ((acc[0].value() + acc[1].value()) + (acc[2].value() + acc[3].value()));
   }
 }
 
-__global__ void __launch_bounds__(NT) k_hxc_fwd_plane(GridPlan gp, const double* __restrict__ rho,
-                                                      c128* __restrict__ scratch, const c128* __restrict__ twg) {
-  extern __shared__ unsigned char smem_raw[];
-  c128* tw = reinterpret_cast<c128*>(smem_raw);
-  c128* buf = tw + 3 * kMaxDim;
-  const int z = blockIdx.x;
-  const int nx = gp.nx, ny = gp.ny, pitch = gp.pitch_x;
-  const int plane = nx * ny;
-  for (int t = threadIdx.x; t < nx + ny + gp.nz; t += NT) tw[t] = twg[t];
-  const double* f = rho + size_t(z) * plane;
-  for (int e = threadIdx.x; e < plane; e += NT) {
-    const int y = e / nx, x = e - y * nx;
-    buf[y * pitch + x] = c128{f[e], 0.0};
+// half: [z][y][kx <= nx/2]; rows 2 p and 2 p + 1 of plane z as one complex line
+__global__ void __launch_bounds__(NT) k_hxc_x_fwd(GridPlan gp, const double* __restrict__ rho, c128* __restrict__ half,
+                                                  const c128* __restrict__ twg) {
+  __shared__ c128 tw[kMaxDim];
+  __shared__ c128 buf[XL * (kMaxDim + 1)];
+  const int z = blockIdx.y, nx = gp.nx, ny = gp.ny, hx = nx / 2 + 1, pitch = gp.pitch_x;
+  const int y0 = blockIdx.x * XL * 2;
+  for (int t = threadIdx.x; t < nx; t += NT) tw[t] = twg[t];
+  const double* f = rho + (size_t(z) * ny + y0) * nx;
+  for (int e = threadIdx.x; e < XL * nx; e += NT) {
+    const int l = e / nx, x = e - l * nx, y = y0 + 2 * l;
+    buf[l * pitch + x] = c128{y < ny ? f[size_t(2 * l) * nx + x] : 0.0, y + 1 < ny ? f[size_t(2 * l + 1) * nx + x] : 0.0};
   }
   __syncthreads();
-  fft_lines<false, NT, MAXE>(buf, gp.ax[0], ny, pitch, 1, tw);
-  fft_lines<false, NT, MAXE>(buf, gp.ax[1], nx, 1, pitch, tw + nx);
-  c128* o = scratch + size_t(z) * plane;
-  for (int e = threadIdx.x; e < plane; e += NT) {
-    const int y = e / nx, x = e - y * nx;
-    o[e] = buf[y * pitch + x];
+  fft_lines<false, NT, XL * kMaxDim>(buf, gp.ax[0], XL, pitch, 1, tw);
+  c128* o = half + (size_t(z) * ny + y0) * hx;
+  for (int e = threadIdx.x; e < XL * hx; e += NT) {
+    const int l = e / hx, k = e - l * hx, y = y0 + 2 * l;
+    const c128 u = buf[l * pitch + k], v = buf[l * pitch + (k ? nx - k : 0)];
+    // the spectra of the two real rows: Hermitian and anti-Hermitian parts
+    if (y < ny) o[size_t(2 * l) * hx + k] = c128{0.5 * (u.re + v.re), 0.5 * (u.im - v.im)};
+    if (y + 1 < ny) o[size_t(2 * l + 1) * hx + k] = c128{0.5 * (u.im + v.im), 0.5 * (v.re - u.re)};
   }
 }
 
-__global__ void __launch_bounds__(NT) k_hxc_column(GridPlan gp, c128* __restrict__ scratch,
-                                                   const double* __restrict__ g2, double inv_ng,
-                                                   const c128* __restrict__ twg) {
-  extern __shared__ unsigned char smem_raw[];
-  c128* tw = reinterpret_cast<c128*>(smem_raw);
-  c128* buf = tw + 3 * kMaxDim;
-  const int yrow = blockIdx.x;
-  const int nx = gp.nx, ny = gp.ny, nz = gp.nz, pitch = gp.pitch_x;
-  for (int t = threadIdx.x; t < nx + ny + nz; t += NT) tw[t] = twg[t];
-  const int slab = nz * nx;
-  for (int e = threadIdx.x; e < slab; e += NT) {
-    const int z = e / nx, x = e - z * nx;
-    buf[z * pitch + x] = scratch[(size_t(z) * ny + yrow) * nx + x];
+// y lines of the half spectrum in place
+template <bool INV>
+__global__ void __launch_bounds__(NT) k_hxc_y(GridPlan gp, c128* __restrict__ half, const c128* __restrict__ twg) {
+  __shared__ c128 tw[kMaxDim];
+  __shared__ c128 buf[CP * kMaxDim];
+  const int ny = gp.ny, hx = gp.nx / 2 + 1, k0 = blockIdx.x * CL, cols = min(CL, hx - k0);
+  for (int t = threadIdx.x; t < ny; t += NT) tw[t] = twg[gp.nx + t];
+  c128* f = half + size_t(blockIdx.y) * ny * hx + k0;
+  for (int e = threadIdx.x; e < CL * ny; e += NT) {
+    const int y = e / CL, c = e % CL;
+    if (c < cols) buf[y * CP + c] = f[size_t(y) * hx + c];
   }
   __syncthreads();
-  fft_lines<false, NT, MAXE>(buf, gp.ax[2], nx, 1, pitch, tw + nx + ny);
-  const double* g2x = g2;
-  const double* g2y = g2 + nx;
-  const double* g2z = g2 + nx + ny;
-  for (int e = threadIdx.x; e < slab; e += NT) {
-    const int z = e / nx, x = e - z * nx;
-    const double G2 = g2x[x] + g2y[yrow] + g2z[z];
-    const double k = G2 > 0.0 ? 4.0 * kPi / G2 * inv_ng : 0.0;
-    buf[z * pitch + x] = buf[z * pitch + x] * k;
-  }
-  __syncthreads();
-  fft_lines<true, NT, MAXE>(buf, gp.ax[2], nx, 1, pitch, tw + nx + ny);
-  for (int e = threadIdx.x; e < slab; e += NT) {
-    const int z = e / nx, x = e - z * nx;
-    scratch[(size_t(z) * ny + yrow) * nx + x] = buf[z * pitch + x];
+  fft_lines<INV, NT, CL * kMaxDim>(buf, gp.ax[1], cols, 1, CP, tw);
+  for (int e = threadIdx.x; e < CL * ny; e += NT) {
+    const int y = e / CL, c = e % CL;
+    if (c < cols) f[size_t(y) * hx + c] = buf[y * CP + c];
   }
 }
 
-// inverse y/x transforms of a plane, LDA, V_loc; optional per-plane energy sums part[2 z + {0, 1}]
-__global__ void __launch_bounds__(NT) k_hxc_inv_plane(GridPlan gp, const c128* __restrict__ scratch,
-                                                      const double* __restrict__ rho, const double* __restrict__ vloc,
-                                                      double* __restrict__ vout, double* __restrict__ part,
-                                                      const c128* __restrict__ twg) {
-  extern __shared__ unsigned char smem_raw[];
-  c128* tw = reinterpret_cast<c128*>(smem_raw);
-  c128* buf = tw + 3 * kMaxDim;
+// z lines: forward, times 4 pi/|G|^2 / Ng, inverse, in place
+__global__ void __launch_bounds__(NT) k_hxc_z(GridPlan gp, c128* __restrict__ half, const double* __restrict__ g2,
+                                              double inv_ng, const c128* __restrict__ twg) {
+  __shared__ c128 tw[kMaxDim];
+  __shared__ c128 buf[CP * kMaxDim];
+  const int nx = gp.nx, ny = gp.ny, nz = gp.nz, hx = nx / 2 + 1, y = blockIdx.y;
+  const int k0 = blockIdx.x * CL, cols = min(CL, hx - k0);
+  for (int t = threadIdx.x; t < nz; t += NT) tw[t] = twg[nx + ny + t];
+  c128* f = half + size_t(y) * hx + k0;
+  for (int e = threadIdx.x; e < CL * nz; e += NT) {
+    const int z = e / CL, c = e % CL;
+    if (c < cols) buf[z * CP + c] = f[size_t(z) * ny * hx + c];
+  }
+  __syncthreads();
+  fft_lines<false, NT, CL * kMaxDim>(buf, gp.ax[2], cols, 1, CP, tw);
+  for (int e = threadIdx.x; e < CL * nz; e += NT) {
+    const int z = e / CL, c = e % CL;
+    if (c >= cols) continue;
+    const double G2 = g2[k0 + c] + g2[nx + y] + g2[nx + ny + z];
+    buf[z * CP + c] = buf[z * CP + c] * (G2 > 0.0 ? 4.0 * kPi / G2 * inv_ng : 0.0);
+  }
+  __syncthreads();
+  fft_lines<true, NT, CL * kMaxDim>(buf, gp.ax[2], cols, 1, CP, tw);
+  for (int e = threadIdx.x; e < CL * nz; e += NT) {
+    const int z = e / CL, c = e % CL;
+    if (c < cols) f[size_t(z) * ny * hx + c] = buf[z * CP + c];
+  }
+}
+
+// inverse x lines (two rows per complex line), LDA, V_loc; optional energy sums of the CTA's rows, part[2 cta + {0, 1}]
+__global__ void __launch_bounds__(NT) k_hxc_x_inv(GridPlan gp, const c128* __restrict__ half, const double* __restrict__ rho,
+                                                  const double* __restrict__ vloc, double* __restrict__ vout,
+                                                  double* __restrict__ part, const c128* __restrict__ twg) {
+  __shared__ c128 tw[kMaxDim];
+  __shared__ c128 buf[XL * (kMaxDim + 1)];
   __shared__ double red[2][NT / 32];
-  const int z = blockIdx.x;
-  const int nx = gp.nx, ny = gp.ny, pitch = gp.pitch_x;
-  const int plane = nx * ny;
-  for (int t = threadIdx.x; t < nx + ny + gp.nz; t += NT) tw[t] = twg[t];
-  const c128* f = scratch + size_t(z) * plane;
-  for (int e = threadIdx.x; e < plane; e += NT) {
-    const int y = e / nx, x = e - y * nx;
-    buf[y * pitch + x] = f[e];
+  const int z = blockIdx.y, nx = gp.nx, ny = gp.ny, hx = nx / 2 + 1, pitch = gp.pitch_x;
+  const int y0 = blockIdx.x * XL * 2;
+  for (int t = threadIdx.x; t < nx; t += NT) tw[t] = twg[t];
+  const c128* f = half + (size_t(z) * ny + y0) * hx;
+  for (int e = threadIdx.x; e < XL * hx; e += NT) {
+    const int l = e / hx, k = e - l * hx, y = y0 + 2 * l;
+    const c128 a = y < ny ? f[size_t(2 * l) * hx + k] : czero<double>();
+    const c128 b = y + 1 < ny ? f[size_t(2 * l + 1) * hx + k] : czero<double>();
+    buf[l * pitch + k] = c128{a.re - b.im, a.im + b.re};                     // a + i b
+    if (k && 2 * k != nx) buf[l * pitch + nx - k] = c128{a.re + b.im, b.re - a.im};  // conj(a) + i conj(b)
   }
   __syncthreads();
-  fft_lines<true, NT, MAXE>(buf, gp.ax[1], nx, 1, pitch, tw + nx);
-  fft_lines<true, NT, MAXE>(buf, gp.ax[0], ny, pitch, 1, tw);
-  const size_t off = size_t(z) * plane;
+  fft_lines<true, NT, XL * kMaxDim>(buf, gp.ax[0], XL, pitch, 1, tw);
+  const size_t off = (size_t(z) * ny + y0) * nx;
+  const int rows = min(2 * XL, ny - y0);
   double eh = 0.0, exc = 0.0;
-  for (int e = threadIdx.x; e < plane; e += NT) {
-    const int y = e / nx, x = e - y * nx;
-    const double vh = buf[y * pitch + x].re;
+  for (int e = threadIdx.x; e < rows * nx; e += NT) {
+    const int q = e / nx, x = e - q * nx;
+    const c128 w = buf[(q >> 1) * pitch + x];
+    const double vh = q & 1 ? w.im : w.re;
     const double r = rho[off + e];
     double eps, vxc;
     lda_point(r, eps, vxc);
@@ -176,27 +218,20 @@ __global__ void __launch_bounds__(NT) k_hxc_inv_plane(GridPlan gp, const c128* _
     red[1][w] = exc;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
-    for (int k = 0; k < NT / 32; ++k) {
-      a += red[0][k];
-      b += red[1][k];
-    }
-    part[2 * z] = a;
-    part[2 * z + 1] = b;
+  if (threadIdx.x < 2) {
+    double a = 0.0;
+    for (int k = 0; k < NT / 32; ++k) a += red[threadIdx.x][k];
+    part[2 * (size_t(z) * gridDim.x + blockIdx.x) + threadIdx.x] = a;
   }
 }
 
-size_t tile_bytes() { return size_t(kMaxDim) * (kMaxDim + 1) * sizeof(c128) + 3 * kMaxDim * sizeof(c128); }
-
-void set_attrs() {
-  static DeviceOnce once;
-  once([] {
-    const int b = int(tile_bytes());
-    PT_CUDA_CHECK(cudaFuncSetAttribute(k_hxc_fwd_plane, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
-    PT_CUDA_CHECK(cudaFuncSetAttribute(k_hxc_column, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
-    PT_CUDA_CHECK(cudaFuncSetAttribute(k_hxc_inv_plane, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
-  });
+// out[2 z + {0, 1}]: the sums of plane z's CTAs
+__global__ void k_hxc_energy(const double* __restrict__ part, int per_plane, int nz, double* __restrict__ out) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= 2 * nz) return;
+  double a = 0.0;
+  for (int k = 0; k < per_plane; ++k) a += part[2 * (size_t(e >> 1) * per_plane + k) + (e & 1)];
+  out[e] = a;
 }
 
 }  // namespace
@@ -217,14 +252,18 @@ void hxc_potential(pt_ctx* ctx, const double* rho, const double* vloc, const pt_
                    cudaStream_t st) {
   const FftTables& ft = fft_tables(ctx, g, PT_FP64);
   const size_t ng = ng_of(g);
-  c128* scratch = static_cast<c128*>(ctx->get("hxc_scratch", ng * sizeof(c128)));
-  set_attrs();
-  const size_t smem = tile_bytes();
+  const int hx = g.nx / 2 + 1, xc = (g.ny + 2 * XL - 1) / (2 * XL), cc = (hx + CL - 1) / CL;
+  // the half spectrum, and per-CTA energy sums
+  const size_t nh = size_t(hx) * g.ny * g.nz;
+  c128* half = static_cast<c128*>(ctx->get("hxc_scratch", nh * sizeof(c128) + 2 * size_t(xc) * g.nz * sizeof(double)));
+  double* sums = part ? reinterpret_cast<double*>(half + nh) : nullptr;
   const c128* tw = static_cast<const c128*>(ft.tw);
-  PT_LAUNCH(k_hxc_fwd_plane, g.nz, NT, smem, st, ft.plan, rho, scratch, tw);
-  PT_LAUNCH(k_hxc_column, g.ny, NT, smem, st, ft.plan, scratch, static_cast<const double*>(ft.g2d),
-            1.0 / double(ng), tw);
-  PT_LAUNCH(k_hxc_inv_plane, g.nz, NT, smem, st, ft.plan, scratch, rho, vloc, v, part, tw);
+  PT_LAUNCH(k_hxc_x_fwd, dim3(xc, g.nz), NT, 0, st, ft.plan, rho, half, tw);
+  PT_LAUNCH(k_hxc_y<false>, dim3(cc, g.nz), NT, 0, st, ft.plan, half, tw);
+  PT_LAUNCH(k_hxc_z, dim3(cc, g.ny), NT, 0, st, ft.plan, half, static_cast<const double*>(ft.g2d), 1.0 / double(ng), tw);
+  PT_LAUNCH(k_hxc_y<true>, dim3(cc, g.nz), NT, 0, st, ft.plan, half, tw);
+  PT_LAUNCH(k_hxc_x_inv, dim3(xc, g.nz), NT, 0, st, ft.plan, half, rho, vloc, v, sums, tw);
+  if (part) PT_LAUNCH(k_hxc_energy, (2 * g.nz + 127) / 128, 128, 0, st, sums, xc, g.nz, part);
 }
 
 }  // namespace pt
