@@ -20,8 +20,10 @@ namespace pt {
 namespace {
 
 constexpr int FT = 256;  // threads per CTA of the tile kernels
-constexpr int AT = 256;  // threads per CTA of the accumulate kernel
-constexpr int AE = 4;    // elements per thread of the accumulate kernel
+constexpr int AT = 128;  // threads per CTA of the accumulate kernel
+constexpr int AE = 1;    // elements per thread of the accumulate kernel
+constexpr int TG = 4;    // targets per CTA of the accumulate kernel
+constexpr int CH = 32;   // contributions per target that it holds at a time
 
 template <int N, class T>
 constexpr size_t tile_smem() {
@@ -124,39 +126,104 @@ __global__ void __launch_bounds__(FT) k_fx_inv_plane(cx<T>* __restrict__ scratch
   }
 }
 
-// W_t(r) -= sum_c d_c partner_c(r) v_c(r)  (v conjugated for the mirrored half of a symmetric pair)
+__device__ __forceinline__ float flip_sign(float x, unsigned m) { return __uint_as_float(__float_as_uint(x) ^ m); }
+__device__ __forceinline__ double flip_sign(double x, unsigned m) {
+  return __longlong_as_double(__double_as_longlong(x) ^ ((long long)(m) << 32));
+}
+
+__device__ __forceinline__ bool same_bits(float a, float b) { return __float_as_uint(a) == __float_as_uint(b); }
+__device__ __forceinline__ bool same_bits(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
+
+// W_t(r) -= sum_c d_c partner_c(r) v_c(r)  (v conjugated for the mirrored half of a symmetric pair) for TG targets of
+// the batch: targets of one tile take their partners in the same order, so d_c partner_c is formed once for them.  In
+// FP64 bound by arithmetic (an instruction issues every 64 cycles): six and a half operations per contribution and
+// point, signs and the test for d = 0 in integers (eight and a comparison with one target to a CTA).
 template <class T>
 __global__ void __launch_bounds__(AT) k_fx_accumulate(const cx<T>* __restrict__ scratch, const cx<T>* __restrict__ src,
                                                       const double* __restrict__ occ,
-                                                      const TargetDesc* __restrict__ tgts,
+                                                      const TargetDesc* __restrict__ tgts, int nt,
                                                       const Contrib* __restrict__ contribs, cx<T>* __restrict__ out,
                                                       size_t ng) {
-  const TargetDesc td = tgts[blockIdx.y];
+  // the contribution lists in shared memory, CH at a time: no chain of dependent loads (list, occupation, field) per
+  // contribution
+  struct Item {
+    int slot, partner;  // slot < 0: no contribution (a skipped pair left its scratch field unwritten)
+    unsigned flip;
+  };
+  __shared__ Item list[TG][CH];
+  __shared__ T coef[TG][CH];
+  const int t0 = blockIdx.y * TG;
+  int most = 0;
+#pragma unroll
+  for (int u = 0; u < TG; ++u)
+    if (t0 + u < nt) most = max(most, tgts[t0 + u].cend - tgts[t0 + u].cbeg);
   const size_t e0 = size_t(blockIdx.x) * (AT * AE) + threadIdx.x;
-  cx<T> acc[AE];
+  cx<T> acc[TG][AE], part[AE];
 #pragma unroll
-  for (int u = 0; u < AE; ++u) acc[u] = czero<T>();
-  for (int c = td.cbeg; c < td.cend; ++c) {
-    const Contrib cb = contribs[c];
-    const T coef = T(occ[cb.occ]);
-    if (coef == T(0)) continue;  // a skipped pair left its scratch field unwritten
-    const cx<T>* v = scratch + size_t(cb.slot) * ng;
-    const cx<T>* pp = src + size_t(cb.partner) * ng;
+  for (int u = 0; u < TG; ++u)
 #pragma unroll
-    for (int u = 0; u < AE; ++u) {
-      const size_t e = e0 + size_t(u) * AT;
-      if (e < ng) {
-        cx<T> w = v[e];
-        if (cb.conj) w.im = -w.im;
-        acc[u] = acc[u] + cmul(pp[e], w) * coef;
+    for (int a = 0; a < AE; ++a) acc[u][a] = czero<T>();
+#pragma unroll
+  for (int a = 0; a < AE; ++a) part[a] = czero<T>();
+  int held = -1;  // the partner in part, with its coefficient
+  T held_coef = T(0);
+  for (int c0 = 0; c0 < most; c0 += CH) {
+    __syncthreads();
+    for (int f = threadIdx.x; f < TG * CH; f += AT) {
+      const int u = f / CH, c = c0 + f % CH;
+      Item it{-1, 0, 0};
+      if (t0 + u < nt) {
+        const TargetDesc td = tgts[t0 + u];
+        if (td.cbeg + c < td.cend) {
+          const Contrib cb = contribs[td.cbeg + c];
+          const double d = occ[cb.occ];
+          if ((__double_as_longlong(d) << 1) != 0) it = Item{cb.slot, cb.partner, cb.conj ? 0x80000000u : 0u};
+          coef[u][f % CH] = T(d);
+        }
+      }
+      list[u][f % CH] = it;
+    }
+    __syncthreads();
+    for (int c = 0; c < min(CH, most - c0); ++c) {
+      cx<T> w[TG][AE];
+#pragma unroll
+      for (int u = 0; u < TG; ++u)
+#pragma unroll
+        for (int a = 0; a < AE; ++a) {
+          const size_t e = e0 + size_t(a) * AT;
+          w[u][a] = (list[u][c].slot >= 0 && e < ng) ? scratch[size_t(list[u][c].slot) * ng + e] : czero<T>();
+        }
+#pragma unroll
+      for (int u = 0; u < TG; ++u) {
+        const Item it = list[u][c];
+        if (it.slot < 0) continue;
+        const T d = coef[u][c];
+        if (it.partner != held || !same_bits(d, held_coef)) {
+          held = it.partner;
+          held_coef = d;
+          const cx<T>* pp = src + size_t(it.partner) * ng;
+#pragma unroll
+          for (int a = 0; a < AE; ++a)
+            if (e0 + size_t(a) * AT < ng) part[a] = pp[e0 + size_t(a) * AT] * d;
+        }
+#pragma unroll
+        for (int a = 0; a < AE; ++a) {
+          w[u][a].im = flip_sign(w[u][a].im, it.flip);
+          acc[u][a] = acc[u][a] + cmul(part[a], w[u][a]);  // one rounding at the sum's size per contribution
+        }
       }
     }
   }
-  cx<T>* o = out + size_t(td.t) * ng;
 #pragma unroll
-  for (int u = 0; u < AE; ++u) {
-    const size_t e = e0 + size_t(u) * AT;
-    if (e < ng) o[e] = td.first ? czero<T>() - acc[u] : o[e] - acc[u];
+  for (int u = 0; u < TG; ++u) {
+    if (t0 + u >= nt) continue;
+    const TargetDesc td = tgts[t0 + u];
+    cx<T>* o = out + size_t(td.t) * ng;
+#pragma unroll
+    for (int a = 0; a < AE; ++a) {
+      const size_t e = e0 + size_t(a) * AT;
+      if (e < ng) o[e] = td.first ? czero<T>() - acc[u][a] : o[e] - acc[u][a];
+    }
   }
 }
 
@@ -185,7 +252,7 @@ void batch_n(const cx<T>* src, const cx<T>* tgt, const double* occ, const PairDe
   PT_LAUNCH((k_fx_column<N, T>), dim3(N, np), FT, smem, st, scratch, ktab, occ, pairs, tw);
   PT_LAUNCH((k_fx_inv_plane<N, T>), dim3(N, np), FT, smem, st, scratch, occ, pairs, tw);
   const unsigned chunks = unsigned((NG + AT * AE - 1) / (AT * AE));
-  PT_LAUNCH(k_fx_accumulate<T>, dim3(chunks, nt), AT, 0, st, scratch, src, occ, tgts, contribs, out, NG);
+  PT_LAUNCH(k_fx_accumulate<T>, dim3(chunks, (nt + TG - 1) / TG), AT, 0, st, scratch, src, occ, tgts, nt, contribs, out, NG);
 }
 
 }  // namespace

@@ -89,53 +89,54 @@ __device__ __forceinline__ cx<T> twiddle(cx<T> a) {
 }
 
 // p + rot90(q) and p - rot90(q)
-template <bool INV>
-__device__ __forceinline__ void cross(c64 p, c64 q, c64& a, c64& b) {
-  const c64 r = rot90<INV>(q);
+template <bool INV, class T>
+__device__ __forceinline__ void cross(cx<T> p, cx<T> q, cx<T>& a, cx<T>& b) {
+  const cx<T> r = rot90<INV>(q);
   a = p + r;
   b = p - r;
 }
 // p + rot90(q) h and p - rot90(q) h
-template <bool INV>
-__device__ __forceinline__ void cross(c64 p, c64 q, float h, c64& a, c64& b) {
-  const float s = INV ? h : -h;
-  a = c64{fmaf(-s, q.im, p.re), fmaf(s, q.re, p.im)};
-  b = c64{fmaf(s, q.im, p.re), fmaf(-s, q.re, p.im)};
+template <bool INV, class T>
+__device__ __forceinline__ void cross(cx<T> p, cx<T> q, T h, cx<T>& a, cx<T>& b) {
+  const T s = INV ? h : -h;
+  a = cx<T>{fma(-s, q.im, p.re), fma(s, q.re, p.im)};
+  b = cx<T>{fma(s, q.im, p.re), fma(-s, q.re, p.im)};
 }
-template <bool INV>
-__device__ __forceinline__ void pdft4(c64& a0, c64& a1, c64& a2, c64& a3) {
-  const c64 s0 = padd(a0, a2), s1 = psub(a0, a2), s2 = padd(a1, a3), s3 = psub(a1, a3);
+template <bool INV, class T>
+__device__ __forceinline__ void pdft4(cx<T>& a0, cx<T>& a1, cx<T>& a2, cx<T>& a3) {
+  const cx<T> s0 = padd(a0, a2), s1 = psub(a0, a2), s2 = padd(a1, a3), s3 = psub(a1, a3);
   a0 = padd(s0, s2);
   a2 = psub(s0, s2);
   cross<INV>(s1, s3, a1, a3);
 }
-template <int R, bool INV>
-__device__ __forceinline__ void pdft(c64* a) {
+// the DFTs of fft.cuh with packed (FP32) and fused operations
+template <int R, bool INV, class T>
+__device__ __forceinline__ void pdft(cx<T>* a) {
   if constexpr (R == 2) {
-    const c64 t = psub(a[0], a[1]);
+    const cx<T> t = psub(a[0], a[1]);
     a[0] = padd(a[0], a[1]);
     a[1] = t;
   } else if constexpr (R == 3) {
-    const c64 s = padd(a[1], a[2]), d = psub(a[1], a[2]), t = pfma(s, -0.5f, a[0]);
+    const cx<T> s = padd(a[1], a[2]), d = psub(a[1], a[2]), t = pfma(s, T(-0.5), a[0]);
     a[0] = padd(a[0], s);
-    cross<INV>(t, d, 0.86602540378443864676f, a[1], a[2]);
+    cross<INV>(t, d, T(0.86602540378443864676), a[1], a[2]);
   } else if constexpr (R == 4) {
     pdft4<INV>(a[0], a[1], a[2], a[3]);
   } else if constexpr (R == 5) {
-    constexpr float c1 = 0.30901699437494742410f, c2 = -0.80901699437494742410f;
-    constexpr float s1 = 0.95105651629515357212f, s2 = 0.58778525229247312917f;
-    const c64 t1 = padd(a[1], a[4]), t2 = padd(a[2], a[3]), d1 = psub(a[1], a[4]), d2 = psub(a[2], a[3]);
-    const c64 b1 = pfma(t2, c2, pfma(t1, c1, a[0])), b2 = pfma(t2, c1, pfma(t1, c2, a[0]));
-    const c64 e1 = pfma(d2, s2, pmul(d1, s1)), e2 = pfma(d2, -s1, pmul(d1, s2));
+    constexpr T c1 = T(0.30901699437494742410), c2 = T(-0.80901699437494742410);
+    constexpr T s1 = T(0.95105651629515357212), s2 = T(0.58778525229247312917);
+    const cx<T> t1 = padd(a[1], a[4]), t2 = padd(a[2], a[3]), d1 = psub(a[1], a[4]), d2 = psub(a[2], a[3]);
+    const cx<T> b1 = pfma(t2, c2, pfma(t1, c1, a[0])), b2 = pfma(t2, c1, pfma(t1, c2, a[0]));
+    const cx<T> e1 = pfma(d2, s2, pmul(d1, s1)), e2 = pfma(d2, -s1, pmul(d1, s2));
     a[0] = padd(padd(a[0], t1), t2);
     cross<INV>(b1, e1, a[1], a[4]);
     cross<INV>(b2, e2, a[2], a[3]);
   } else {
-    constexpr float r = 0.70710678118654752440f;
-    c64 e0 = a[0], e1 = a[2], e2 = a[4], e3 = a[6], o0 = a[1], o1 = a[3], o2 = a[5], o3 = a[7];
+    constexpr T r = T(0.70710678118654752440);
+    cx<T> e0 = a[0], e1 = a[2], e2 = a[4], e3 = a[6], o0 = a[1], o1 = a[3], o2 = a[5], o3 = a[7];
     pdft4<INV>(e0, e1, e2, e3);
     pdft4<INV>(o0, o1, o2, o3);
-    const c64 p1 = o1 + rot90<INV>(o1), p3 = rot90<INV>(o3) - o3;
+    const cx<T> p1 = o1 + rot90<INV>(o1), p3 = rot90<INV>(o3) - o3;
     a[0] = padd(e0, o0);
     a[4] = psub(e0, o0);
     a[1] = pfma(p1, r, e1);
@@ -198,8 +199,7 @@ __device__ __forceinline__ void short_dft(cx<T>* a) {
   else if constexpr (R == 10) pair_dft<2, 5, INV>(a);
   else if constexpr (R == 12) pair_dft<3, 4, INV>(a);
   else if constexpr (R == 16) pair_dft<4, 4, INV>(a);
-  else if constexpr (sizeof(T) == 4) pdft<R, INV>(a);
-  else dft<R, INV>(a);
+  else pdft<R, INV>(a);
 }
 
 // the split of a line length: the shorter factor first, coprime where the length allows it

@@ -30,5 +30,10 @@ __device__ __forceinline__ c64 pmul(c64 a, float s) {
       : "f"(a.re), "f"(a.im), "f"(s));
   return r;
 }
+// the same operations in FP64, one component at a time
+__device__ __forceinline__ c128 padd(c128 a, c128 b) { return a + b; }
+__device__ __forceinline__ c128 psub(c128 a, c128 b) { return a - b; }
+__device__ __forceinline__ c128 pfma(c128 a, double s, c128 c) { return {fma(a.re, s, c.re), fma(a.im, s, c.im)}; }
+__device__ __forceinline__ c128 pmul(c128 a, double s) { return a * s; }
 }  // namespace rl
 }  // namespace pt
