@@ -66,44 +66,74 @@ __device__ __forceinline__ void jacobi_pair(int k, int r, int Np, int* p, int* q
   *q = max(a, b);
 }
 
+template <class T>
 struct Rot {
-  double c, s;
-  c128 u;  // J = [[c, s u], [-s conj(u), c]]
+  T c, s;
+  cx<T> u;  // J = [[c, s u], [-s conj(u), c]]
 };
 
-// the rotation that annihilates a_pq, or the identity (s = 0) when |a_pq|^2 <= thr2 (threshold
-// Jacobi: an entry already below the stopping level is left in place)
-__device__ __forceinline__ Rot jacobi_rot(const c128* A, int N, int p, int q, double thr2) {
-  Rot r{1.0, 0.0, c128{1.0, 0.0}};
-  if (q >= N) return r;  // padding player
-  const c128 apq = A[size_t(p) * N + q];
-  const double b2 = apq.re * apq.re + apq.im * apq.im;
+__device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
+
+// the rotation that annihilates apq (diagonal entries app, aqq), or the identity (s = 0) when |a_pq|^2 <= thr2
+// (threshold Jacobi: an entry already below the stopping level is left in place)
+template <class T>
+__device__ __forceinline__ Rot<T> jacobi_angle(cx<T> apq, T app, T aqq, T thr2) {
+  Rot<T> r{T(1), T(0), cx<T>{T(1), T(0)}};
+  const T b2 = apq.re * apq.re + apq.im * apq.im;
   if (!(b2 > thr2)) return r;
-  const double app = A[size_t(p) * N + p].re, aqq = A[size_t(q) * N + q].re;
   // reciprocal square roots in place of square roots and divisions (each a long FP64 sequence on
   // the round's critical path)
-  const double rb = rsqrt(b2);  // 1 / |a_pq|
-  const double zeta = (aqq - app) * (0.5 * rb);
-  const double az = fabs(zeta);
-  double t;
-  if (az > 1e100) {
-    t = 0.5 / az;  // 1 / (|zeta| + sqrt(1 + zeta^2)) to double precision
+  const T rb = rsq(b2);  // 1 / |a_pq|
+  const T zeta = (aqq - app) * (T(0.5) * rb);
+  const T az = fabs(zeta);
+  T t;
+  if (az > (sizeof(T) == 8 ? T(1e100) : T(1e15f))) {
+    t = T(0.5) / az;  // 1 / (|zeta| + sqrt(1 + zeta^2)) to working precision
   } else {
-    const double q2 = 1.0 + zeta * zeta;
-    t = 1.0 / (az + q2 * rsqrt(q2));
+    const T q2 = T(1) + zeta * zeta;
+    t = T(1) / (az + q2 * rsq(q2));
   }
-  if (zeta < 0.0) t = -t;
-  r.c = rsqrt(1.0 + t * t);
+  if (zeta < T(0)) t = -t;
+  r.c = rsq(T(1) + t * t);
   r.s = t * r.c;
-  r.u = c128{apq.re * rb, apq.im * rb};
+  r.u = cx<T>{apq.re * rb, apq.im * rb};
   return r;
+}
+template <class T>
+__device__ __forceinline__ Rot<T> jacobi_rot(const cx<T>* A, int N, int p, int q, T thr2) {
+  if (q >= N) return Rot<T>{T(1), T(0), cx<T>{T(1), T(0)}};  // padding player
+  return jacobi_angle(A[size_t(p) * N + q], A[size_t(p) * N + p].re, A[size_t(q) * N + q].re, thr2);
+}
+
+// Z = J_a^H X J_b of a 2 x 2 block; same: the block that the rotation diagonalises
+template <class T>
+__device__ __forceinline__ void rotate_block(const Rot<T>& a, const Rot<T>& b, bool same, cx<T>& x00, cx<T>& x01,
+                                             cx<T>& x10, cx<T>& x11) {
+  // Y = J_a^H X:  J^H = [[c, -s u], [s conj(u), c]]
+  const cx<T> su = a.u * a.s, suc = conjc(a.u) * a.s;
+  const cx<T> y00 = x00 * a.c - cmul(su, x10), y01 = x01 * a.c - cmul(su, x11);
+  const cx<T> y10 = cmul(suc, x00) + x10 * a.c, y11 = cmul(suc, x01) + x11 * a.c;
+  // Z = Y J_b:  J = [[c, s u], [-s conj(u), c]]
+  const cx<T> tu = b.u * b.s, tuc = conjc(b.u) * b.s;
+  x00 = y00 * b.c - cmul(y01, tuc);
+  x01 = cmul(y00, tu) + y01 * b.c;
+  x10 = y10 * b.c - cmul(y11, tuc);
+  x11 = cmul(y10, tu) + y11 * b.c;
+  if (same) {
+    x01 = czero<T>();
+    x10 = czero<T>();
+    x00.im = T(0);
+    x11.im = T(0);
+  }
 }
 
 constexpr int JB = 8;  // pairs per CTA side (16 x 16 elements): (N/16)^2 CTAs spread over every SM
 
-__global__ void __launch_bounds__(JB* JB) k_jacobi_round(const c128* __restrict__ Ain, c128* __restrict__ Aout,
-                                                         c128* __restrict__ V, int N, int Np, int r, double thr2) {
-  __shared__ Rot rk[JB], rl[JB];
+template <class T>
+__global__ void __launch_bounds__(JB* JB) k_jacobi_round(const cx<T>* __restrict__ Ain, cx<T>* __restrict__ Aout,
+                                                         cx<T>* __restrict__ V, int N, int Np, int r, T thr2) {
+  __shared__ Rot<T> rk[JB], rl[JB];
   __shared__ int pk[JB], qk[JB], pl[JB], ql[JB];
   const int kb = blockIdx.y * JB, lb = blockIdx.x * JB;
   const int half = Np / 2;
@@ -128,34 +158,22 @@ __global__ void __launch_bounds__(JB* JB) k_jacobi_round(const c128* __restrict_
   const int k = kb + tk, l = lb + tl;
   if (k < half && l < half) {
     const int p1 = pk[tk], q1 = qk[tk], p2 = pl[tl], q2 = ql[tl];
-    const Rot a = rk[tk], b = rl[tl];
-    auto get = [&](int i, int j) -> c128 {
-      return (i < N && j < N) ? Ain[size_t(i) * N + j] : czero<double>();
+    const Rot<T> a = rk[tk], b = rl[tl];
+    auto get = [&](int i, int j) -> cx<T> {
+      return (i < N && j < N) ? Ain[size_t(i) * N + j] : czero<T>();
     };
-    const c128 x00 = get(p1, p2), x01 = get(p1, q2), x10 = get(q1, p2), x11 = get(q1, q2);
-    auto put = [&](int i, int j, c128 v) {
+    const cx<T> x00 = get(p1, p2), x01 = get(p1, q2), x10 = get(q1, p2), x11 = get(q1, q2);
+    auto put = [&](int i, int j, cx<T> v) {
       if (i < N && j < N) Aout[size_t(i) * N + j] = v;
     };
-    if (a.s == 0.0 && b.s == 0.0) {  // both rotations the identity: the block is carried over
+    if (a.s == T(0) && b.s == T(0)) {  // both rotations the identity: the block is carried over
       put(p1, p2, x00);
       put(p1, q2, x01);
       put(q1, p2, x10);
       put(q1, q2, x11);
     } else {
-      // Y = J_a^H X:  J^H = [[c, -s u], [s conj(u), c]]
-      const c128 su = a.u * a.s, suc = conjc(a.u) * a.s;
-      const c128 y00 = x00 * a.c - cmul(su, x10), y01 = x01 * a.c - cmul(su, x11);
-      const c128 y10 = cmul(suc, x00) + x10 * a.c, y11 = cmul(suc, x01) + x11 * a.c;
-      // Z = Y J_b:  J = [[c, s u], [-s conj(u), c]]
-      const c128 tu = b.u * b.s, tuc = conjc(b.u) * b.s;
-      c128 z00 = y00 * b.c - cmul(y01, tuc), z01 = cmul(y00, tu) + y01 * b.c;
-      c128 z10 = y10 * b.c - cmul(y11, tuc), z11 = cmul(y10, tu) + y11 * b.c;
-      if (k == l) {  // the 2x2 block this rotation diagonalises
-        z01 = czero<double>();
-        z10 = czero<double>();
-        z00.im = 0.0;
-        z11.im = 0.0;
-      }
+      cx<T> z00 = x00, z01 = x01, z10 = x10, z11 = x11;
+      rotate_block(a, b, k == l, z00, z01, z10, z11);
       put(p1, p2, z00);
       put(p1, q2, z01);
       put(q1, p2, z10);
@@ -173,14 +191,218 @@ __global__ void __launch_bounds__(JB* JB) k_jacobi_round(const c128* __restrict_
       if (l2 >= half) continue;
       const int p2 = pl[tl2], q2 = ql[tl2];
       if (q2 >= N) continue;
-      const Rot b = rl[tl2];
-      if (b.s == 0.0) continue;  // identity
-      const c128 vp = V[size_t(row) * N + p2], vq = V[size_t(row) * N + q2];
-      const c128 tu = b.u * b.s, tuc = conjc(b.u) * b.s;
+      const Rot<T> b = rl[tl2];
+      if (b.s == T(0)) continue;  // identity
+      const cx<T> vp = V[size_t(row) * N + p2], vq = V[size_t(row) * N + q2];
+      const cx<T> tu = b.u * b.s, tuc = conjc(b.u) * b.s;
       V[size_t(row) * N + p2] = vp * b.c - cmul(vq, tuc);
       V[size_t(row) * N + q2] = cmul(vp, tu) + vq * b.c;
     }
   }
+}
+
+// ---- FP32 Jacobi on D + E --------------------------------------------------------------------------------------
+//
+// The off-diagonal part E in FP32, the diagonal D as unevaluated pairs of floats (48 bits), so that differences of
+// close eigenvalues are exact: a pass lowers E by FP32's relative precision (~1e-6) however small E already is,
+// and finds a basis that is accurate to that times E. Two passes, each made unitary in FP64 and followed by
+// X^* A X in FP64, take a matrix from anywhere to 1e-12 of its norm.
+
+// the rotation of (p, q) from E and D; D is updated in place by the owner of the pair
+__device__ __forceinline__ Rot<float> jacobi32_angle(c64 apq, float2 dp, float2 dq, float thr2) {
+  return jacobi_angle(apq, 0.f, (dq.x - dp.x) + (dq.y - dp.y), thr2);
+}
+__device__ __forceinline__ float2 pair_add(float2 a, float b) {  // two-sum
+  const float s = __fadd_rn(a.x, b), v = __fsub_rn(s, a.x);
+  const float e = __fadd_rn(__fadd_rn(__fsub_rn(a.x, __fsub_rn(s, v)), __fsub_rn(b, v)), a.y);
+  const float h = __fadd_rn(s, e);
+  return make_float2(h, __fsub_rn(e, __fsub_rn(h, s)));
+}
+__device__ __forceinline__ float2 to_pair(double x) {
+  const float h = float(x);
+  return make_float2(h, float(x - double(h)));
+}
+// app -> app - t |apq|, aqq -> aqq + t |apq| with t = s / c
+__device__ __forceinline__ void rotate_diag(const Rot<float>& r, c64 apq, float2& dp, float2& dq) {
+  if (r.s == 0.f) return;
+  const float d = (r.s / r.c) * (apq.re * r.u.re + apq.im * r.u.im);
+  dp = pair_add(dp, -d);
+  dq = pair_add(dq, d);
+}
+
+// when to stop: off and off0 the off-diagonal norms^2 now and at the start, prev after the sweep before
+__host__ __device__ inline bool jacobi32_done(double off, double off0, double prev, double floor2, int N) {
+  return !(off > floor2) || off <= 1e-14 * N * off0 || (off <= 1e-9 * off0 && off > 0.25 * prev);
+}
+
+// One CTA, E and the basis in shared memory (N <= J32_MAX): whole sweeps, two barriers a round (0.7 us at N = 48 against
+// 8.7 us of k_jacobi_round, which is a launch and a chain of FP64 instructions).  X: the basis, as FP64.
+constexpr int J32_MAX = 96, J32_THREADS = 1024;
+constexpr size_t j32_smem(int N) { return 2 * size_t(N) * (N | 1) * sizeof(c64); }
+__global__ void __launch_bounds__(J32_THREADS) k_jacobi32_cta(const c128* __restrict__ A, int N, float floor2,
+                                                              c128* __restrict__ X) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int P = N | 1, Np = N + (N & 1), half = Np / 2;
+  c64* a = reinterpret_cast<c64*>(smem_raw);
+  c64* v = a + size_t(N) * P;
+  __shared__ Rot<float> rot[J32_MAX / 2];
+  __shared__ short2 pq[J32_MAX / 2];
+  __shared__ float2 dg[J32_MAX];
+  __shared__ float red[J32_THREADS / 32];
+  const int t = threadIdx.x;
+  for (int e = t; e < N * N; e += J32_THREADS) {
+    const int i = e / N, j = e - i * N;
+    if (i == j) dg[i] = to_pair(A[e].re);
+    a[i * P + j] = to_cx<float>(A[e]);
+    v[i * P + j] = c64{i == j ? 1.f : 0.f, 0.f};
+  }
+  float prev = INFINITY, off0 = 0.f, thr2 = 0.f;
+  for (int sweep = 0; sweep < 12; ++sweep) {
+    __syncthreads();
+    float off = 0.f;
+    for (int e = t; e < N * N; e += J32_THREADS) {
+      const int i = e / N, j = e - i * N;
+      const c64 x = a[i * P + j];
+      if (i != j) off += x.re * x.re + x.im * x.im;
+    }
+    for (int o = 16; o; o >>= 1) off += __shfl_xor_sync(0xffffffffu, off, o);
+    if ((t & 31) == 0) red[t >> 5] = off;
+    __syncthreads();
+    off = 0.f;
+    for (int w = 0; w < J32_THREADS / 32; ++w) off += red[w];
+    if (sweep == 0) {
+      off0 = off;
+      thr2 = fmaxf(1e-15f * off0, floor2) / (float(N) * float(N));
+    }
+    // uniform: every thread added the same sums
+    if (sweep > 0 && jacobi32_done(off, off0, prev, floor2, N)) break;
+    if (sweep > 0) prev = off;
+    for (int r = 0; r < Np - 1; ++r) {
+      __syncthreads();
+      if (t < half) {
+        int p, q;
+        jacobi_pair(t, r, Np, &p, &q);
+        pq[t] = make_short2(short(p), short(q));
+        Rot<float> x{1.f, 0.f, c64{1.f, 0.f}};
+        if (q < N) {
+          const c64 apq = a[p * P + q];
+          x = jacobi32_angle(apq, dg[p], dg[q], thr2);
+          rotate_diag(x, apq, dg[p], dg[q]);
+        }
+        rot[t] = x;
+      }
+      __syncthreads();
+      for (int e = t; e < half * half; e += J32_THREADS) {
+        const int k = e / half, l = e - k * half;
+        const Rot<float> x = rot[k], y = rot[l];
+        if (x.s == 0.f && y.s == 0.f) continue;
+        const int p1 = pq[k].x, q1 = pq[k].y, p2 = pq[l].x, q2 = pq[l].y;
+        if (k == l) {
+          a[p1 * P + q1] = a[q1 * P + p1] = czero<float>();
+          continue;
+        }
+        const bool in1 = q1 < N, in2 = q2 < N;
+        c64 x00 = a[p1 * P + p2], x01 = in2 ? a[p1 * P + q2] : czero<float>();
+        c64 x10 = in1 ? a[q1 * P + p2] : czero<float>(), x11 = in1 && in2 ? a[q1 * P + q2] : czero<float>();
+        rotate_block(x, y, false, x00, x01, x10, x11);
+        a[p1 * P + p2] = x00;
+        if (in2) a[p1 * P + q2] = x01;
+        if (in1) a[q1 * P + p2] = x10;
+        if (in1 && in2) a[q1 * P + q2] = x11;
+      }
+      for (int e = t; e < N * half; e += J32_THREADS) {
+        const int row = e / half, l = e - row * half;
+        const Rot<float> y = rot[l];
+        const int p = pq[l].x, q = pq[l].y;
+        if (y.s == 0.f || q >= N) continue;
+        const c64 vp = v[row * P + p], vq = v[row * P + q], tu = y.u * y.s, tuc = conjc(y.u) * y.s;
+        v[row * P + p] = vp * y.c - cmul(vq, tuc);
+        v[row * P + q] = cmul(vp, tu) + vq * y.c;
+      }
+    }
+  }
+  __syncthreads();
+  for (int e = t; e < N * N; e += J32_THREADS) {
+    const c64 x = v[(e / N) * P + e % N];
+    X[e] = c128{double(x.re), double(x.im)};
+  }
+}
+
+// The same round over the whole GPU (larger N): E from Ein to Eout, D from Din to Dout, V in place
+__global__ void __launch_bounds__(JB* JB) k_jacobi32_round(const c64* __restrict__ Ein, c64* __restrict__ Eout,
+                                                           const float2* __restrict__ Din, float2* __restrict__ Dout,
+                                                           c64* __restrict__ V, int N, int Np, int r, float thr2) {
+  __shared__ Rot<float> rot[2][JB];
+  __shared__ int pp[2][JB], qq[2][JB];
+  const int kb = blockIdx.y * JB, lb = blockIdx.x * JB, half = Np / 2, t = threadIdx.x;
+  pdl_wait();  // the previous round
+  pdl_launch_dependents();
+  if (t < 2 * JB) {
+    const int side = t / JB, i = t % JB, k = (side ? lb : kb) + i;
+    if (k < half) {
+      int p, q;
+      jacobi_pair(k, r, Np, &p, &q);
+      pp[side][i] = p;
+      qq[side][i] = q;
+      Rot<float> x{1.f, 0.f, c64{1.f, 0.f}};
+      const bool owner = kb == lb && side == 0;
+      if (q < N) {
+        const c64 apq = Ein[size_t(p) * N + q];
+        float2 dp = Din[p], dq = Din[q];
+        x = jacobi32_angle(apq, dp, dq, thr2);
+        if (owner) {
+          rotate_diag(x, apq, dp, dq);
+          Dout[p] = dp;
+          Dout[q] = dq;
+        }
+      } else if (owner) {
+        Dout[p] = Din[p];
+      }
+      rot[side][i] = x;
+    }
+  }
+  __syncthreads();
+  const int tk = t / JB, tl = t % JB, k = kb + tk, l = lb + tl;
+  if (k < half && l < half) {
+    const int p1 = pp[0][tk], q1 = qq[0][tk], p2 = pp[1][tl], q2 = qq[1][tl];
+    const Rot<float> x = rot[0][tk], y = rot[1][tl];
+    const bool in1 = q1 < N, in2 = q2 < N;
+    c64 x00 = Ein[size_t(p1) * N + p2], x01 = in2 ? Ein[size_t(p1) * N + q2] : czero<float>();
+    c64 x10 = in1 ? Ein[size_t(q1) * N + p2] : czero<float>(), x11 = in1 && in2 ? Ein[size_t(q1) * N + q2] : czero<float>();
+    if (x.s != 0.f || y.s != 0.f) {
+      if (k == l) x01 = x10 = czero<float>();
+      else rotate_block(x, y, false, x00, x01, x10, x11);
+    }
+    Eout[size_t(p1) * N + p2] = x00;
+    if (in2) Eout[size_t(p1) * N + q2] = x01;
+    if (in1) Eout[size_t(q1) * N + p2] = x10;
+    if (in1 && in2) Eout[size_t(q1) * N + q2] = x11;
+  }
+  // V <- V J for this CTA's l range, the rows split over the CTAs of that range
+  const int rows = (N + gridDim.y - 1) / gridDim.y, r0 = blockIdx.y * rows, r1 = min(N, r0 + rows);
+  for (int e = t; e < (r1 - r0) * JB; e += JB * JB) {
+    const int row = r0 + e / JB, i = e % JB;
+    if (lb + i >= half || qq[1][i] >= N || rot[1][i].s == 0.f) continue;
+    const Rot<float> y = rot[1][i];
+    c64 *vp = V + size_t(row) * N + pp[1][i], *vq = V + size_t(row) * N + qq[1][i];
+    const c64 a = *vp, b = *vq, tu = y.u * y.s, tuc = conjc(y.u) * y.s;
+    *vp = a * y.c - cmul(b, tuc);
+    *vq = cmul(a, tu) + b * y.c;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_jacobi32_start(const c128* __restrict__ A, int N, c64* __restrict__ E,
+                                                        float2* __restrict__ D, c64* __restrict__ V) {
+  const int e = blockIdx.x * 256 + threadIdx.x;
+  if (e >= N * N) return;
+  const int i = e / N, j = e - i * N;
+  E[e] = i == j ? czero<float>() : to_cx<float>(A[e]);
+  if (i == j) D[i] = to_pair(A[e].re);
+  V[e] = c64{i == j ? 1.f : 0.f, 0.f};
+}
+__global__ void __launch_bounds__(256) k_widen(const c64* __restrict__ V32, int n, c128* __restrict__ X) {
+  const int e = blockIdx.x * 256 + threadIdx.x;
+  if (e < n) X[e] = c128{double(V32[e].re), double(V32[e].im)};
 }
 
 // A = (S + S^*)/2 and V = V0 (identity when V0 is NULL)
@@ -197,11 +419,12 @@ __global__ void k_herm_part_and_basis(const c128* __restrict__ S, c128* __restri
 // sums of |offdiag|^2 and |all|^2: one partial pair per block (OFF_BLOCKS blocks), then one thread
 // adds the partials in order
 constexpr int OFF_BLOCKS = 64;
-__global__ void __launch_bounds__(256) k_offnorm_part(const c128* __restrict__ A, int N, double* __restrict__ part) {
+template <class T>
+__global__ void __launch_bounds__(256) k_offnorm_part(const cx<T>* __restrict__ A, int N, double* __restrict__ part) {
   pdl_wait();  // the last Jacobi round
   double off = 0, all = 0;
   for (int e = blockIdx.x * 256 + threadIdx.x; e < N * N; e += OFF_BLOCKS * 256) {
-    const double v = A[e].re * A[e].re + A[e].im * A[e].im;
+    const double v = double(A[e].re) * double(A[e].re) + double(A[e].im) * double(A[e].im);
     all += v;
     if (e / N != e % N) off += v;
   }
@@ -273,9 +496,6 @@ __global__ void k_eig_permute(const c128* __restrict__ V, const int* __restrict_
 // factored (and inverted) in one CTA's shared memory, the panel below is solved against the
 // inverse of the diagonal block, and the trailing lower triangle gets a rank-CB update.
 constexpr int CB = 32;
-
-__device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
 
 template <class T>
 __global__ void __launch_bounds__(256) k_chol_diag(cx<T>* __restrict__ A, int N, int kb, int bs,
@@ -509,14 +729,74 @@ int heev(pt_ctx* ctx, const c128* S, int N, c128* Q, double* d, cudaStream_t st,
   const int half = Np / 2;
   dim3 grid((half + JB - 1) / JB, (half + JB - 1) / JB);
   double h[2] = {0, 0};
-  double prev_off = INFINITY;
-  int sweeps = 0;
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    PT_LAUNCH_PDL(k_offnorm_part, OFF_BLOCKS, 256, 0, st, A0, N, nrm + 2);
+  auto norms = [&](auto* A) {
+    PT_LAUNCH_PDL((k_offnorm_part<std::decay_t<decltype(A->re)>>), OFF_BLOCKS, 256, 0, st, A, N, nrm + 2);
     PT_LAUNCH(k_offnorm_sum, 1, 32, 0, st, nrm + 2, nrm);
     PT_CUDA_CHECK(cudaMemcpyAsync(h, nrm, sizeof(h), cudaMemcpyDeviceToHost, st));
     PT_CUDA_CHECK(cudaStreamSynchronize(st));
     if (!std::isfinite(h[1])) fail(PT_NONFINITE, "non-finite entry in the matrix to diagonalise");
+  };
+  // Where the caller asks for less than FP64 rounding (rel_tol): FP32 passes on D + E (see k_jacobi32_cta), each basis
+  // made unitary in FP64 by two Newton-Schulz steps (X <- X (3 I - X^* X)/2, the error squared each time) and
+  // A <- X^* A X in FP64.  Two passes usually meet the tolerance, whose test stays that of the FP64 sweeps below, which
+  // finish the rest.  A pass costs seven FP64 products and its sweeps (N = 48: 2.05 -> 0.80 ms a solve; N = 320, a launch
+  // per FP32 round: 25 -> 15 ms).
+  for (int pass = 0; rel_tol > 0.0 && pass < 3; ++pass) {
+    const double before = h[0];
+    norms(A0);
+    const double floor2 = 0.01 * rel_tol * rel_tol * h[1];
+    if (!(h[1] > 1e-6 && h[1] < 1e12) || h[0] <= rel_tol * rel_tol * h[1]) break;
+    if (pass > 0 && h[0] > 1e-4 * before) break;  // no longer gaining: leave it to the FP64 sweeps
+    c128* X0 = static_cast<c128*>(ctx->get("heev_X0", size_t(N) * N * sizeof(c128)));
+    c128* X1 = static_cast<c128*>(ctx->get("heev_X1", size_t(N) * N * sizeof(c128)));
+    c128* G = static_cast<c128*>(ctx->get("heev_G", size_t(N) * N * sizeof(c128)));
+    const int nb = (N * N + 255) / 256;
+    if (N <= J32_MAX) {
+      static DeviceOnce once;
+      once([] {
+        PT_CUDA_CHECK(
+            cudaFuncSetAttribute(k_jacobi32_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, int(j32_smem(J32_MAX))));
+      });
+      PT_LAUNCH(k_jacobi32_cta, 1, J32_THREADS, j32_smem(N), st, A0, N, float(floor2), X0);
+    } else {
+      // E and V in buffers that are free until the products below
+      c64 *e0 = reinterpret_cast<c64*>(G), *e1 = e0 + size_t(N) * N, *v32 = reinterpret_cast<c64*>(X1);
+      float2* d0 = static_cast<float2*>(ctx->get("heev_D32", 2 * size_t(N) * sizeof(float2)));
+      float2* d1 = d0 + N;
+      PT_LAUNCH(k_jacobi32_start, nb, 256, 0, st, A0, N, e0, d0, v32);
+      const double off0 = h[0];
+      const float thr2 = float(std::max(1e-15 * off0, floor2) / (double(N) * double(N)));
+      double prev = INFINITY;
+      for (int sweep = 0; sweep < 12; ++sweep) {
+        if (sweep > 0) {
+          norms(e0);
+          if (jacobi32_done(h[0], off0, prev, floor2, N)) break;
+          prev = h[0];
+        }
+        for (int r = 0; r < Np - 1; ++r) {
+          PT_LAUNCH_PDL(k_jacobi32_round, grid, JB * JB, 0, st, e0, e1, d0, d1, v32, N, Np, r, thr2);
+          std::swap(e0, e1);
+          std::swap(d0, d1);
+        }
+      }
+      h[0] = off0;
+      PT_LAUNCH(k_widen, nb, 256, 0, st, v32, N * N, X0);
+    }
+    const c128 one{1, 0}, zero{0, 0};
+    for (int it = 0; it < 2; ++it) {
+      zgemm('C', 'N', N, N, N, one, X0, N, X0, N, zero, G, N, st);
+      zgemm_add('N', 'N', N, N, N, c128{-0.5, 0}, X0, N, G, N, c128{1.5, 0}, X0, N, X1, N, st);
+      std::swap(X0, X1);
+    }
+    zgemm('N', 'N', N, N, N, one, A0, N, X0, N, zero, G, N, st);
+    zgemm('C', 'N', N, N, N, one, X0, N, G, N, zero, A1, N, st);
+    zgemm('N', 'N', N, N, N, one, V, N, X0, N, zero, G, N, st);
+    PT_LAUNCH(k_herm_part_and_basis, nb, 256, 0, st, A1, A0, G, V, N);
+  }
+  double prev_off = INFINITY;
+  int sweeps = 0;
+  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
+    norms(A0);
     // Converged when the off-diagonal norm is at the FP64 rounding floor (eps * sqrt(N) * ||A||),
     // or when, already small, a sweep no longer reduces it (cyclic Jacobi converges
     // quadratically, so a stalled sweep means rounding noise).
@@ -531,7 +811,7 @@ int heev(pt_ctx* ctx, const c128* S, int N, c128* Q, double* d, cudaStream_t st,
     const double stop2 = rel_tol > 0.0 ? rel_tol * rel_tol * h[1] : floor2;
     const double thr2 = std::max(1e-280, stop2 / (double(N) * double(N)));
     for (int r = 0; r < Np - 1; ++r) {
-      PT_LAUNCH_PDL(k_jacobi_round, grid, JB * JB, 0, st, A0, A1, V, N, Np, r, thr2);
+      PT_LAUNCH_PDL(k_jacobi_round<double>, grid, JB * JB, 0, st, A0, A1, V, N, Np, r, thr2);
       std::swap(A0, A1);
     }
     ++sweeps;
