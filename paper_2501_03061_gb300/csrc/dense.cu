@@ -57,6 +57,43 @@ __global__ void __launch_bounds__(ZT* ZT) k_gemm(char opA, char opB, int m, int 
   }
 }
 
+// The same for small matrices: 8 x 8 tiles with the k range over four groups of threads.  An FP64 instruction issues every 64
+// cycles per SM sub-partition, so a 16 x 16 tile of a 48 x 48 product kept 9 of 152 SMs busy for 12 us.
+constexpr int ST = 8, SG = 4;
+template <class T>
+__global__ void __launch_bounds__(ST* ST* SG) k_gemm_small(char opA, char opB, int m, int n, int k, cx<T> alpha,
+                                                           const cx<T>* __restrict__ A, int lda, const cx<T>* __restrict__ B,
+                                                           int ldb, cx<T> beta, const cx<T>* D, int ldd, cx<T>* C, int ldc) {
+  constexpr int KS = 32;  // k per stage
+  __shared__ cx<T> As[ST][KS + 1];
+  __shared__ cx<T> Bs[KS][ST + 1];
+  __shared__ cx<T> red[SG - 1][ST * ST];
+  const int t = threadIdx.x, e = t % (ST * ST), g = t / (ST * ST), ty = e / ST, tx = e % ST;
+  const int i0 = blockIdx.y * ST, j0 = blockIdx.x * ST, i = i0 + ty, j = j0 + tx;
+  cx<T> acc = czero<T>();
+  for (int k0 = 0; k0 < k; k0 += KS) {
+    for (int f = t; f < ST * KS; f += ST * ST * SG) {
+      // consecutive threads on consecutive addresses of op(A) and op(B)
+      const int r = opA == 'N' ? f / KS : f % ST, c = opA == 'N' ? f % KS : f / ST;
+      As[r][c] = (i0 + r < m && k0 + c < k) ? opval(A, lda, opA, i0 + r, k0 + c) : czero<T>();
+      const int q = opB == 'N' ? f / ST : f % KS, l = opB == 'N' ? f % ST : f / KS;
+      Bs[q][l] = (k0 + q < k && j0 + l < n) ? opval(B, ldb, opB, k0 + q, j0 + l) : czero<T>();
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < KS / SG; ++kk)
+      if (k0 + g * (KS / SG) + kk < k) cfma(acc, As[ty][g * (KS / SG) + kk], Bs[g * (KS / SG) + kk][tx]);
+    __syncthreads();
+  }
+  if (g > 0) red[g - 1][e] = acc;
+  __syncthreads();
+  if (g > 0 || i >= m || j >= n) return;
+  for (int q = 0; q < SG - 1; ++q) acc = acc + red[q][e];
+  cx<T> v = cmul(alpha, acc);
+  if (beta.re != T(0) || beta.im != T(0)) v = v + cmul(beta, D[size_t(i) * ldd + j]);
+  C[size_t(i) * ldc + j] = v;
+}
+
 // ---------------------------------------------------------------- Jacobi ----
 // pair partner of position k in round r of the circle method on Np (even) players
 __device__ __forceinline__ void jacobi_pair(int k, int r, int Np, int* p, int* q) {
@@ -497,15 +534,32 @@ __global__ void k_eig_permute(const c128* __restrict__ V, const int* __restrict_
 // inverse of the diagonal block, and the trailing lower triangle gets a rank-CB update.
 constexpr int CB = 32;
 
+// a positive finite number, tested on its bits (an FP64 comparison issues at the FP64 rate here)
+__device__ __forceinline__ bool good_pivot(float x) {
+  const int b = __float_as_int(x);
+  return b > 0 && b < 0x7f800000;
+}
+__device__ __forceinline__ bool good_pivot(double x) {
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b < 0x7ff0000000000000ll;
+}
+
+// Factor and inverse of a diagonal block as A = U D U^* (U unit lower triangular): step k subtracts column k's outer product
+// from the trailing triangle and column k from the rows of U^{-1} below it; L = U D^{1/2} and L^{-1} = D^{-1/2} U^{-1}
+// at the end.  A step is one barrier: warp 0 updates the next pivot and forms its reciprocal while the other
+// warps do the rest, so the FP64 chain (six dependent operations and a reciprocal) and the FP64 work run side by
+// side.  (With a square root, the column and the update behind barriers of their own and the inverse row by row after
+// them a 32 x 32 FP64 block took 95 us; this takes 52.)
 template <class T>
 __global__ void __launch_bounds__(256) k_chol_diag(cx<T>* __restrict__ A, int N, int kb, int bs,
                                                    cx<T>* __restrict__ Winv, int* __restrict__ info) {
   __shared__ cx<T> a[CB][CB + 1];
   __shared__ cx<T> x[CB][CB + 1];
   // lower triangle (i >= j) listed column by column: entry (j, i) at j*bs - j(j-1)/2 + (i - j), so
-  // the trailing triangle of step k (j > k) is one contiguous range and no thread idles on the
-  // upper half
+  // the trailing triangle of step k (j > k) is one contiguous range, its first entry the next pivot
   __shared__ unsigned short tri[CB * (CB + 1) / 2];
+  __shared__ T rd[CB], rs[CB];  // reciprocals of the pivots and of their square roots
+  __shared__ int bad;
   pdl_wait();  // the previous panel's trailing update
   pdl_launch_dependents();
   if (*info) return;
@@ -513,64 +567,54 @@ __global__ void __launch_bounds__(256) k_chol_diag(cx<T>* __restrict__ A, int N,
   for (int e = tid; e < bs * bs; e += blockDim.x) {
     const int i = e / bs, j = e % bs;
     a[i][j] = A[size_t(kb + i) * N + kb + j];
+    x[i][j] = cx<T>{T(i == j ? 1 : 0), T(0)};
     if (i >= j) tri[j * bs - j * (j - 1) / 2 + (i - j)] = static_cast<unsigned short>((j << 8) | i);
   }
   __syncthreads();
+  auto pivot = [&](int k) {  // one thread: a[k][k] is final
+    const T d = a[k][k].re;
+    if (good_pivot(d)) rd[k] = T(1) / d;
+    else bad = k + 1;
+  };
+  if (tid == 0) {
+    bad = 0;
+    pivot(0);
+  }
+  __syncthreads();
   const int tri_end = bs * (bs + 1) / 2;
-  // FP64 square roots and divisions are long instruction sequences on the FP64 pipe: one thread
-  // takes them and broadcasts the results
-  __shared__ T rdiag[CB];
-  __shared__ T s_rk;
   for (int k = 0; k < bs; ++k) {
-    const T piv = a[k][k].re;
-    if (!(piv > 0.0) || !isfinite(piv)) {
-      if (tid == 0) *info = kb + k + 1;
-      return;  // uniform: every thread read the same pivot
+    if (bad) {  // uniform: read behind the barrier that followed its writing
+      if (tid == 0) *info = kb + bad;
+      return;
     }
-    __syncthreads();
-    if (tid == 0) {
-      // one reciprocal square root instead of a square root and a division (each a long FP64
-      // sequence on the pivot's critical path)
-      const T rk0 = rsq(piv);
-      a[k][k] = cx<T>{piv * rk0, T(0)};
-      s_rk = rk0;
-      rdiag[k] = rk0;
-    }
-    __syncthreads();
-    const T rk = s_rk;
-    for (int i = k + 1 + tid; i < bs; i += blockDim.x) a[i][k] = a[i][k] * rk;
-    __syncthreads();
-    for (int e = (k + 1) * bs - (k + 1) * k / 2 + tid; e < tri_end; e += blockDim.x) {
-      const int i = tri[e] & 255, j = tri[e] >> 8;
-      a[i][j] = a[i][j] - cmulc(a[j][k], a[i][k]);
-    }
-    __syncthreads();
-  }
-  // inverse X of the lower-triangular factor, one row at a time with all threads:
-  //   X[i][i] = 1 / L[i][i],  X[i][j] = -(sum_{p=j}^{i-1} L[i][p] X[p][j]) / L[i][i]  (j < i);
-  // thread (part, j) sums every 8th p, the 8 parts meet in shared memory
-  __shared__ cx<T> red[8][CB];
-  {
-    const int j = tid & (CB - 1), part = tid >> 5;
-    for (int i = 0; i < bs; ++i) {
-      cx<T> acc = czero<T>();
-      if (j < i)
-        for (int p = j + part; p < i; p += 8) acc = acc + cmul(a[i][p], x[p][j]);
-      red[part][j] = acc;
-      __syncthreads();
-      if (part == 0) {
-        cx<T> t = czero<T>();
-        for (int q = 0; q < 8; ++q) t = t + red[q][j];
-        const T inv = rdiag[i];
-        x[i][j] = j < i ? t * (-inv) : (j == i ? cx<T>{inv, T(0)} : czero<T>());
+    const T r = rd[k];
+    const int first = (k + 1) * bs - (k + 1) * k / 2;
+    if (tid < 32) {
+      if (tid == 0 && k + 1 < bs) {
+        const cx<T> c = a[k + 1][k];
+        a[k + 1][k + 1].re -= (c.re * c.re + c.im * c.im) * r;
+        pivot(k + 1);
       }
-      __syncthreads();
+    } else {
+      const int n1 = max(0, tri_end - first - 1), n2 = (bs - 1 - k) * (k + 1);
+      for (int e = tid - 32; e < n1 + n2; e += 256 - 32) {
+        if (e < n1) {
+          const int i = tri[first + 1 + e] & 255, j = tri[first + 1 + e] >> 8;
+          a[i][j] = a[i][j] - cmulc(a[j][k] * r, a[i][k]);
+        } else {
+          const int f = e - n1, i = k + 1 + f / (k + 1), j = f % (k + 1);
+          x[i][j] = x[i][j] - cmul(a[i][k] * r, x[k][j]);
+        }
+      }
     }
+    __syncthreads();
   }
+  if (tid < bs) rs[tid] = rsq(a[tid][tid].re);
+  __syncthreads();
   for (int e = tid; e < bs * bs; e += blockDim.x) {
     const int i = e / bs, j = e % bs;
-    if (j <= i) A[size_t(kb + i) * N + kb + j] = a[i][j];
-    Winv[i * CB + j] = x[i][j];
+    if (j <= i) A[size_t(kb + i) * N + kb + j] = j == i ? cx<T>{a[i][i].re * rs[i], T(0)} : a[i][j] * rs[j];
+    Winv[i * CB + j] = j <= i ? x[i][j] * rs[i] : czero<T>();
   }
 }
 
@@ -691,6 +735,12 @@ __global__ void k_small_solve(const double* __restrict__ G, const double* __rest
 template <class T>
 void gemm(char opA, char opB, int m, int n, int k, cx<T> alpha, const cx<T>* A, int lda, const cx<T>* B, int ldb,
           cx<T> beta, const cx<T>* D, int ldd, cx<T>* C, int ldc, cudaStream_t st) {
+  // small tiles while 16 x 16 ones would leave SMs idle (152 of them): FP64 N = 48 17.6 -> 9 us a product, N = 75 23 -> 9
+  if (((n + ZT - 1) / ZT) * ((m + ZT - 1) / ZT) < 152) {
+    PT_LAUNCH(k_gemm_small<T>, dim3((n + ST - 1) / ST, (m + ST - 1) / ST), ST * ST * SG, 0, st, opA, opB, m, n, k, alpha, A,
+              lda, B, ldb, beta, D, ldd, C, ldc);
+    return;
+  }
   dim3 grid((n + ZT - 1) / ZT, (m + ZT - 1) / ZT);
   PT_LAUNCH(k_gemm<T>, grid, ZT * ZT, 0, st, opA, opB, m, n, k, alpha, A, lda, B, ldb, beta, D, ldd, C, ldc);
 }
