@@ -12,6 +12,8 @@
 // stage complete (barrier) before any write, so one buffer serves in place.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace pt {
@@ -200,6 +202,23 @@ struct FftTables {
   pt_precision prec;
   ~FftTables();
 };
+
+// Key of a context cache: a name and the bytes of its values (printing five doubles took 3 us of a call)
+struct CacheKey {
+  std::string s;
+  explicit CacheKey(const char* name) : s(name) {}
+  template <class T>
+  CacheKey& operator<<(const T& v) {
+    static_assert(std::is_arithmetic<T>::value, "a number, without padding");
+    s.append(reinterpret_cast<const char*>(&v), sizeof(T));
+    return *this;
+  }
+};
+inline CacheKey grid_cache_key(const char* name, const pt_grid& g) {
+  CacheKey k(name);
+  k << g.nx << g.ny << g.nz << g.L[0] << g.L[1] << g.L[2];
+  return k;
+}
 
 // Tables for (grid, precision) cached in the context.
 const FftTables& fft_tables(pt_ctx* ctx, const pt_grid& g, pt_precision prec);

@@ -81,9 +81,7 @@ static void fill_tables(FftTables* t, const pt_grid& g) {
 
 const FftTables& fft_tables(pt_ctx* ctx, const pt_grid& g, pt_precision prec) {
   const bool dbl = (prec == PT_FP64);
-  char key[160];
-  snprintf(key, sizeof(key), "fft:%d:%d:%d:%.17g:%.17g:%.17g:%d", g.nx, g.ny, g.nz, g.L[0], g.L[1], g.L[2],
-           int(dbl));
+  const std::string key = (grid_cache_key("fft:", g) << int(dbl)).s;
   auto it = ctx->caches.find(key);
   if (it != ctx->caches.end()) return *std::static_pointer_cast<FftTables>(it->second);
   auto t = std::make_shared<FftTables>();
@@ -113,9 +111,7 @@ double kernel_value(const pt_kernel& k, double G2) {
 
 const void* kernel_table(pt_ctx* ctx, const pt_grid& g, const pt_kernel& k, pt_precision prec) {
   const bool dbl = (prec == PT_FP64);
-  char key[200];
-  snprintf(key, sizeof(key), "ktab:%d:%d:%d:%.17g:%.17g:%.17g:%d:%.17g:%.17g:%d", g.nx, g.ny, g.nz, g.L[0],
-           g.L[1], g.L[2], k.type, k.mu, k.g0, int(dbl));
+  const std::string key = (grid_cache_key("ktab:", g) << k.type << k.mu << k.g0 << int(dbl)).s;
   auto it = ctx->caches.find(key);
   if (it != ctx->caches.end()) return std::static_pointer_cast<KernelTableImpl>(it->second)->d;
   const size_t ng = ng_of(g);

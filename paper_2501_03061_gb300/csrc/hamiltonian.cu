@@ -232,8 +232,7 @@ void apply_h(pt_ctx* ctx, const void* psi, int M, void* out, const double* vloc,
 const unsigned long long* sphere_masks(pt_ctx* ctx, const pt_grid& g, const double* g2d, double ecut,
                                        cudaStream_t st) {
   if (g.nx != g.ny || g.nx != g.nz || g.nx > 64) fail(PT_INVALID_ARG, "sphere masks: cubic grids of side <= 64");
-  char key[160];
-  snprintf(key, sizeof(key), "sphere_masks:%d:%.17g:%.17g:%.17g:%.17g", g.nx, g.L[0], g.L[1], g.L[2], ecut);
+  const std::string key = (grid_cache_key("sphere_masks:", g) << ecut).s;
   auto it = ctx->caches.find(key);
   if (it != ctx->caches.end()) return std::static_pointer_cast<SphereMasks>(it->second)->d;
   auto sm = std::make_shared<SphereMasks>();
