@@ -113,16 +113,18 @@ __device__ __forceinline__ void copy_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N));
 }
 
-// FP32 Gram tile of 64 x 64 outputs, 4 x 4 complex per thread, 16 grid points per stage; the
+// FP32 Gram tile of 16 R x 16 R outputs, R x R complex per thread, 16 grid points per stage; the
 // per-stage sums are folded into Kahan-compensated totals.  With herm, only tiles on or above
 // the diagonal run (the reduction mirrors the rest).  Bound by FP32 arithmetic and its issue: the next
 // stage's operands arrive by asynchronous copies while this one is multiplied, and a complex product is
 // two packed instructions.
-constexpr int G4T = 64, G4K = 16, G4THREADS = 256;
+constexpr int G4K = 16, G4THREADS = 256;
 
-__global__ void __launch_bounds__(G4THREADS, 2) k_gram64(const c64* __restrict__ A, const c64* __restrict__ B,
+template <int R>
+__global__ void __launch_bounds__(G4THREADS, 2) k_gram32(const c64* __restrict__ A, const c64* __restrict__ B,
                                                          int N1, int N2, size_t ng, size_t chunk, int herm,
                                                          c128* __restrict__ part) {
+  constexpr int G4T = 16 * R;
   if (herm && blockIdx.y < blockIdx.x) return;
   __shared__ c64 As[2][G4K][G4T + 1];
   __shared__ c64 Bs[2][G4K][G4T + 1];
@@ -143,7 +145,7 @@ __global__ void __launch_bounds__(G4THREADS, 2) k_gram64(const c64* __restrict__
     }
     copy_commit();
   };
-  Acc<float> sre[4][4], sim[4][4];
+  Acc<float> sre[R][R], sim[R][R];
   int buf = 0;
   if (r_begin < r_end) fetch(r_begin, 0);
   for (size_t r0 = r_begin; r0 < r_end; r0 += G4K, buf ^= 1) {
@@ -154,27 +156,27 @@ __global__ void __launch_bounds__(G4THREADS, 2) k_gram64(const c64* __restrict__
       copy_wait<0>();
     }
     __syncthreads();
-    c64 acc[4][4];
+    c64 acc[R][R];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < R; ++a)
 #pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = czero<float>();
+      for (int b = 0; b < R; ++b) acc[a][b] = czero<float>();
 #pragma unroll 4
     for (int k = 0; k < G4K; ++k) {
-      c64 av[4];
+      c64 av[R];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = As[buf][k][ti + 16 * a];
+      for (int a = 0; a < R; ++a) av[a] = As[buf][k][ti + 16 * a];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
+      for (int b = 0; b < R; ++b) {
         const c64 bv = Bs[buf][k][tj + 16 * b], bx = c64{bv.im, -bv.re};  // conj(a) b = Re(a) b + Im(a) (-i b)
 #pragma unroll
-        for (int a = 0; a < 4; ++a) acc[a][b] = rl::pfma(bx, av[a].im, rl::pfma(bv, av[a].re, acc[a][b]));
+        for (int a = 0; a < R; ++a) acc[a][b] = rl::pfma(bx, av[a].im, rl::pfma(bv, av[a].re, acc[a][b]));
       }
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < R; ++a)
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
+      for (int b = 0; b < R; ++b) {
         sre[a][b].add(acc[a][b].re);
         sim[a][b].add(acc[a][b].im);
       }
@@ -182,9 +184,9 @@ __global__ void __launch_bounds__(G4THREADS, 2) k_gram64(const c64* __restrict__
   }
   c128* P = part + size_t(blockIdx.z) * N1 * N2;
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < R; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
+    for (int b = 0; b < R; ++b) {
       const int i = i0 + ti + 16 * a, j = j0 + tj + 16 * b;
       if (i < N1 && j < N2) P[size_t(i) * N2 + j] = c128{sre[a][b].value(), sim[a][b].value()};
     }
@@ -430,19 +432,31 @@ void gram(pt_ctx* ctx, const cx<T>* A, const cx<T>* B, int N1, int N2, size_t ng
     }
   }
   const bool f32 = sizeof(T) == 4;
-  const int tile = f32 ? G4T : GT;
+  // FP32 tile of 64, 48 or 32 orbitals: the one that pads N1 x N2 least (75 x 75 in four tiles of 48 instead of 64: 145 ->
+  // 85 us), the larger where they tie: it reads less per product
+  int R = 4;
+  if (f32) {
+    auto area = [&](int r) { return size_t((N1 + 16 * r - 1) / (16 * r)) * ((N2 + 16 * r - 1) / (16 * r)) * r * r; };
+    for (int r = 3; r >= 2; --r)
+      if (area(r) < area(R)) R = r;
+  }
+  const int tile = f32 ? 16 * R : GT;
   const int kstep = f32 ? G4K : GK;
   herm = herm && (N1 == N2);
   const int ti = (N1 + tile - 1) / tile, tj = (N2 + tile - 1) / tile;
   const int tiles = herm ? ti * (ti + 1) / 2 : ti * tj;
-  // enough splits along r to fill the GPU about four times (two CTAs per SM for the FP32 tile)
-  int splits = std::max(1, (ctx->num_sms * 4 + tiles - 1) / tiles);
+  // enough splits along r to fill the GPU about four times; twice, one wave of the two CTAs per SM, for the FP32 tile
+  // (61 x 61 at 40^3: 68 us with its sum against 77)
+  int splits = std::max(1, (ctx->num_sms * (f32 ? 2 : 4)) / tiles);
   size_t chunk = (ng + splits - 1) / splits;
   chunk = (chunk + kstep - 1) / kstep * kstep;
   splits = int((ng + chunk - 1) / chunk);
   c128* part = static_cast<c128*>(ctx->get("gram_parts", size_t(splits) * N1 * N2 * sizeof(c128)));
   if constexpr (sizeof(T) == 4) {
-    PT_LAUNCH(k_gram64, dim3(ti, tj, splits), G4THREADS, 0, st, A, B, N1, N2, ng, chunk, int(herm), part);
+    const dim3 grid(ti, tj, splits);
+    if (R == 4) PT_LAUNCH(k_gram32<4>, grid, G4THREADS, 0, st, A, B, N1, N2, ng, chunk, int(herm), part);
+    else if (R == 3) PT_LAUNCH(k_gram32<3>, grid, G4THREADS, 0, st, A, B, N1, N2, ng, chunk, int(herm), part);
+    else PT_LAUNCH(k_gram32<2>, grid, G4THREADS, 0, st, A, B, N1, N2, ng, chunk, int(herm), part);
   } else {
     herm = false;
     PT_LAUNCH(k_gram<T>, dim3(ti, tj, splits), GTHREADS, 0, st, A, B, N1, N2, ng, chunk, part);
