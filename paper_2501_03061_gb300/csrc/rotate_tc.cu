@@ -19,9 +19,14 @@
 // copy instead of a tiled load of 2 x 128 rows of 128 bytes.  Products summed per tile:
 // hi*hi + hi*lo + lo*hi.
 //
-// Warp roles (320 threads): warp 0 TMA producer, warp 1 TMEM allocation and MMA issue (one
-// lane), warps 2..5 converter, warps 6..9 TMEM readout and the epilogue (alpha is folded into
-// B'; the epilogue adds the extra terms and stores complex64).  CTAs are persistent and walk
+// Warp roles (448 threads): warp 0 TMA producer, warp 1 TMEM allocation and MMA issue (one
+// lane), warps 2..5 converter, warps 6..9 and 10..13 TMEM readout and epilogue of half of the columns each
+// (alpha is folded into B'; the epilogue adds the extra terms and stores complex64).  B' stages have a
+// ring of their own, three deep, so that their 32 KB copies run ahead of the conversions (with one ring of
+// two for both operands a stage's buffers took the MMAs, the copy and the conversion in turn; 54^3, 200 x 200
+// 512 -> 446 us, 60^3, 150 x 150 434 -> 366, 64^3, 320 x 320 1371 -> 1275).  What bounds it now is shared
+// memory: by count 96 KB of operand reads and 96 KB of copies and conversions a stage, 1500 cycles; two
+// converter warpgroups (96 registers a thread) ran slower, 507 us.  CTAs are persistent and walk
 // the tiles with a grid stride; the two TMEM accumulators alternate between periods, so the
 // epilogue of one tile overlaps the MMAs of the next.  Every wait is bounded (%globaltimer); on
 // expiry the CTA records an error, leaves its loops, drains its own copies and tensor-core work
@@ -40,14 +45,17 @@ constexpr int RJ = 64;                  // output orbitals per tile (MMA N = 2 R
 constexpr int NC = 2 * RJ;              // 128 real output columns
 constexpr int KO = 16;                  // orbitals per K stage (32 floats of K')
 constexpr int RA = 3;                   // raw A stages
-constexpr int RC = 2;                   // converted / B stages
-constexpr int THREADS = 320;
+constexpr int RC = 2;                   // converted A stages
+constexpr int RB = 3;                   // B stages
+constexpr int RO = 2;                   // readout warpgroups (NC / RO columns each)
+constexpr int THREADS = 64 + 128 * (1 + RO);
 constexpr uint32_t RAW_BYTES = KO * RM * 8;          // 16 KB: [16 orbitals][128 points] complex64
 constexpr uint32_t OP_BYTES = 128 * 128;             // 16 KB: 128 rows x 32 floats, swizzled
-constexpr uint32_t CST_BYTES = 4 * OP_BYTES;         // A hi | A lo | B hi | B lo
+constexpr uint32_t CST_BYTES = 2 * OP_BYTES;         // A hi | A lo, or B hi | B lo
 constexpr uint32_t OFF_C = 0;                        // converted ring (1024-aligned stages)
-constexpr uint32_t OFF_RAW = RC * CST_BYTES;         // 131072
-constexpr uint32_t OFF_BAR = OFF_RAW + RA * RAW_BYTES;  // 180224
+constexpr uint32_t OFF_B = RC * CST_BYTES;           // B ring
+constexpr uint32_t OFF_RAW = OFF_B + RB * CST_BYTES;
+constexpr uint32_t OFF_BAR = OFF_RAW + RA * RAW_BYTES;  // 212992
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 256 + 1024;
 constexpr uint64_t TIMEOUT_NS = 2000000000ull;
 
@@ -153,18 +161,21 @@ __global__ void __launch_bounds__(THREADS, 1)
   auto bar_a_full = [&](int s) { return bar0 + 8u * s; };
   auto bar_a_empty = [&](int s) { return bar0 + 8u * (RA + s); };
   auto bar_b_full = [&](int s) { return bar0 + 8u * (2 * RA + s); };
-  auto bar_c_full = [&](int s) { return bar0 + 8u * (2 * RA + RC + s); };
-  auto bar_c_empty = [&](int s) { return bar0 + 8u * (2 * RA + 2 * RC + s); };
-  auto bar_acc_full = [&](int b) { return bar0 + 8u * (2 * RA + 3 * RC + b); };
-  auto bar_acc_empty = [&](int b) { return bar0 + 8u * (2 * RA + 3 * RC + 2 + b); };
-  const uint32_t bar_drain = bar0 + 8u * (2 * RA + 3 * RC + 4);
+  auto bar_b_empty = [&](int s) { return bar0 + 8u * (2 * RA + RB + s); };
+  constexpr int NB = 2 * RA + 2 * RB;
+  auto bar_c_full = [&](int s) { return bar0 + 8u * (NB + s); };
+  auto bar_c_empty = [&](int s) { return bar0 + 8u * (NB + RC + s); };
+  auto bar_acc_full = [&](int b) { return bar0 + 8u * (NB + 2 * RC + b); };
+  auto bar_acc_empty = [&](int b) { return bar0 + 8u * (NB + 2 * RC + 2 + b); };
+  const uint32_t bar_drain = bar0 + 8u * (NB + 2 * RC + 4);
+  static_assert(8 * (NB + 2 * RC + 5) <= 192, "barriers below the TMEM address");
   volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(sm + OFF_BAR + 192);
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(sm + OFF_BAR + 200);
   auto a_raw = [&](int s) { return base + OFF_RAW + uint32_t(s) * RAW_BYTES; };
   auto c_ahi = [&](int s) { return base + OFF_C + uint32_t(s) * CST_BYTES; };
   auto c_alo = [&](int s) { return c_ahi(s) + OP_BYTES; };
-  auto c_bhi = [&](int s) { return c_ahi(s) + 2 * OP_BYTES; };
-  auto c_blo = [&](int s) { return c_ahi(s) + 3 * OP_BYTES; };
+  auto c_bhi = [&](int s) { return base + OFF_B + uint32_t(s) * CST_BYTES; };
+  auto c_blo = [&](int s) { return c_bhi(s) + OP_BYTES; };
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // this CTA's tiles: blockIdx.x, blockIdx.x + gridDim.x, ...
@@ -178,14 +189,17 @@ __global__ void __launch_bounds__(THREADS, 1)
       mbar_init(bar_a_full(s), 1);
       mbar_init(bar_a_empty(s), 128);
     }
-    for (int s = 0; s < RC; ++s) {
+    for (int s = 0; s < RB; ++s) {
       mbar_init(bar_b_full(s), 1);
+      mbar_init(bar_b_empty(s), 1);
+    }
+    for (int s = 0; s < RC; ++s) {
       mbar_init(bar_c_full(s), 128);
       mbar_init(bar_c_empty(s), 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(bar_acc_full(b), 1);
-      mbar_init(bar_acc_empty(b), 128);
+      mbar_init(bar_acc_empty(b), 128 * RO);
     }
     mbar_init(bar_drain, 1);
     *abort_flag = 0;
@@ -219,7 +233,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       for (int q = 0; q < nq && !*abort_flag; ++q) {
         int rb, jt, s;
         tile_of(q, rb, jt, s);
-        const int sa = q % RA, sc = q % RC;
+        const int sa = q % RA, sb = q % RB;
         if (q >= RA && !mbar_wait(bar_a_empty(sa), ((q / RA) - 1) & 1, TIMEOUT_NS)) {
           fail_out(1);
           break;
@@ -227,33 +241,33 @@ __global__ void __launch_bounds__(THREADS, 1)
         mbar_arrive_expect_tx(bar_a_full(sa), RAW_BYTES);
         tma_load_4d(a_raw(sa), &tmA, rb * RM, s * KO, 0, 0, bar_a_full(sa));
         issued_a = q + 1;
-        if (q >= RC && !mbar_wait(bar_c_empty(sc), ((q / RC) - 1) & 1, TIMEOUT_NS)) {
+        if (q >= RB && !mbar_wait(bar_b_empty(sb), ((q / RB) - 1) & 1, TIMEOUT_NS)) {
           fail_out(2);
           break;
         }
-        mbar_arrive_expect_tx(bar_b_full(sc), 2 * OP_BYTES);
-        bulk_load(c_bhi(sc), P.bp + size_t(jt * S + s) * (2 * OP_BYTES / 4), 2 * OP_BYTES, bar_b_full(sc));
+        mbar_arrive_expect_tx(bar_b_full(sb), 2 * OP_BYTES);
+        bulk_load(c_bhi(sb), P.bp + size_t(jt * S + s) * (2 * OP_BYTES / 4), 2 * OP_BYTES, bar_b_full(sb));
         issued_b = q + 1;
       }
       // copies in flight land before the CTA's shared memory is released
       for (int q = max(0, issued_a - RA); q < issued_a; ++q)
         if (!mbar_wait(bar_a_full(q % RA), (q / RA) & 1, TIMEOUT_NS)) atomicOr(err, 128);
-      for (int q = max(0, issued_b - RC); q < issued_b; ++q)
-        if (!mbar_wait(bar_b_full(q % RC), (q / RC) & 1, TIMEOUT_NS)) atomicOr(err, 128);
+      for (int q = max(0, issued_b - RB); q < issued_b; ++q)
+        if (!mbar_wait(bar_b_full(q % RB), (q / RB) & 1, TIMEOUT_NS)) atomicOr(err, 128);
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
       int gp = 0;  // global period counter (selects the TMEM accumulator)
       for (int q = 0; q < nq && !*abort_flag; ++q) {
-        const int s = q % S, sc = q % RC;
+        const int s = q % S, sc = q % RC, sb = q % RB;
         const int b = gp & 1;
         const bool first = (s % P.period) == 0;
         if (first && gp >= 2 && !mbar_wait(bar_acc_empty(b), ((gp / 2) - 1) & 1, TIMEOUT_NS)) {
           fail_out(4);
           break;
         }
-        if (!mbar_wait(bar_b_full(sc), (q / RC) & 1, TIMEOUT_NS) ||
+        if (!mbar_wait(bar_b_full(sb), (q / RB) & 1, TIMEOUT_NS) ||
             !mbar_wait(bar_c_full(sc), (q / RC) & 1, TIMEOUT_NS)) {
           fail_out(8);
           break;
@@ -264,13 +278,14 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (int kk = 0; kk < 4; ++kk) {
           const uint32_t off = uint32_t(kk * 32);
           const uint32_t acc = (first && kk == 0) ? 0u : 1u;
-          mma_tf32(d, smem_desc_sw128(c_ahi(sc) + off), smem_desc_sw128(c_bhi(sc) + off), acc);
+          mma_tf32(d, smem_desc_sw128(c_ahi(sc) + off), smem_desc_sw128(c_bhi(sb) + off), acc);
           if (P.split3) {
-            mma_tf32(d, smem_desc_sw128(c_ahi(sc) + off), smem_desc_sw128(c_blo(sc) + off), 1u);
-            mma_tf32(d, smem_desc_sw128(c_alo(sc) + off), smem_desc_sw128(c_bhi(sc) + off), 1u);
+            mma_tf32(d, smem_desc_sw128(c_ahi(sc) + off), smem_desc_sw128(c_blo(sb) + off), 1u);
+            mma_tf32(d, smem_desc_sw128(c_alo(sc) + off), smem_desc_sw128(c_bhi(sb) + off), 1u);
           }
         }
         mma_commit(bar_c_empty(sc));
+        mma_commit(bar_b_empty(sb));
         if ((s % P.period) == P.period - 1 || s == S - 1) {
           mma_commit(bar_acc_full(b));
           ++gp;
@@ -318,12 +333,14 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int quad = warp & 3;
     const int lrow = 32 * quad + lane;
     const uint32_t lane_base = uint32_t(32 * quad) << 16;
-    float acc[NC];
+    constexpr int CR = NC / RO, JR = RJ / RO;  // this warpgroup's columns and orbitals of the tile
+    const int half = (warp - 6) / 4;
+    float acc[CR];
     int gp = 0;
     bool ok = true;
     for (int t = 0; t < my_tiles && ok; ++t) {
 #pragma unroll
-      for (int c = 0; c < NC; ++c) acc[c] = 0.f;
+      for (int c = 0; c < CR; ++c) acc[c] = 0.f;
       for (int p = 0; p < per_tile; ++p, ++gp) {
         if (__any_sync(0xffffffffu, *abort_flag != 0)) {
           ok = false;
@@ -337,9 +354,9 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         tc_fence_after();
 #pragma unroll
-        for (int c0 = 0; c0 < NC; c0 += 16) {
+        for (int c0 = 0; c0 < CR; c0 += 16) {
           float v[16];
-          tmem_ld16(tmem + lane_base + uint32_t(b * NC + c0), v);
+          tmem_ld16(tmem + lane_base + uint32_t(b * NC + half * CR + c0), v);
 #pragma unroll
           for (int i = 0; i < 16; ++i) acc[c0 + i] += v[i];
         }
@@ -359,14 +376,14 @@ __global__ void __launch_bounds__(THREADS, 1)
         const c64* __restrict__ e1 = P.e[1];
         const c64* __restrict__ e2 = P.e[2];
         c64* __restrict__ op = P.out;
-        const int jn = min(RJ, P.N2 - jt * RJ);
+        const int jb = jt * RJ + half * JR, jn = min(JR, P.N2 - jb);
         // fully unrolled so that acc[] stays in registers
 #pragma unroll
-        for (int j0 = 0; j0 < RJ; j0 += 4) {
+        for (int j0 = 0; j0 < JR; j0 += 4) {
           c64 tv[3][4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const size_t idx = size_t(jt * RJ + j0 + u) * size_t(P.ng) + size_t(r);
+            const size_t idx = size_t(jb + j0 + u) * size_t(P.ng) + size_t(r);
             const bool okj = j0 + u < jn;
             tv[0][u] = (e0 && okj) ? ldg_c64(e0 + idx) : c64{0.f, 0.f};
             tv[1][u] = (e1 && okj) ? ldg_c64(e1 + idx) : c64{0.f, 0.f};
@@ -376,7 +393,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           for (int u = 0; u < 4; ++u) {
             const int jj = j0 + u;
             if (jj >= jn) continue;
-            const size_t idx = size_t(jt * RJ + jj) * size_t(P.ng) + size_t(r);
+            const size_t idx = size_t(jb + jj) * size_t(P.ng) + size_t(r);
             c64 o{acc[2 * jj], acc[2 * jj + 1]};
             o = o + cmul(P.c[0], tv[0][u]) + cmul(P.c[1], tv[1][u]) + cmul(P.c[2], tv[2][u]);
             op[idx] = o;
