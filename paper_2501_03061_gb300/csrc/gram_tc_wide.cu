@@ -12,20 +12,31 @@
 // comes from three TF32 products hi*hi + hi*lo + lo*hi (the raw FP32 value is its own TF32 "hi";
 // "lo" = x - tf32(x) is written by the converter warps).
 //
-// Warp roles (576 threads): warp 0 issues the TMA loads of a stage (A block, half 0, half 1),
-// warp 1 allocates TMEM and one lane issues tcgen05.mma, warps 2..17 (four warpgroups) convert
-// the stage (i*A rows and the lo parts) and read the TMEM accumulator out every `period` stages
-// into Kahan-compensated FP32 registers, each warpgroup owning 32 of the 128 accumulator
-// columns (the TMEM lane quarter of a warp is its index mod 4).  Two TMEM accumulators alternate.
+// Warp roles (640 threads, five warpgroups): one lane of group 0 issues tcgen05.mma; groups 1 and 2 take the
+// stages in turn: they copy them (cp.async), write [A; i A] as hi and lo parts into TMEM, where the MMA reads its A
+// operand, and B's lo parts into shared memory; groups 3 and 4 read the accumulator out every `period` stages
+// into Kahan-compensated FP32 registers, 64 of its 128 columns each.  Two TMEM accumulators alternate; setmaxnreg
+// gives the readout the registers that the other groups do without.
+//   What bounds it: a stage of three products is 770 cycles of MMA, 380 of B operand reads and 600 of copies,
+// conversions and spills on the shared-memory pipe, and takes about 1450; without two of the three products it took
+// 1200, without the conversions or the copies 1400, without most of the readout 1300 (no single one is the wall).  Before, with
+// one TMA-fed ring of 64 KB stages, A in shared memory and 16 warps that converted and read out in turn, it took
+// 1950: boxes of 64 rows of 128 bytes arrive at no more than 31 GB/s a CTA (1500 cycles a stage), A operands
+// were another 380 cycles of reads, and conversion and readout waited for each other.  54^3, 200 x 200: 625 -> 477 us
+// a call, 64^3, 320 x 320 1776 -> 1354, its Hermitian form 1148 -> 884.  A in TMEM alone gave nothing (54^3: 690 in place
+// of 670); a third converter group costs the readout registers (541 against 520), four readout groups of 32
+// columns likewise (562 against 539).
 // The K range of every tile is split over CTAs; each CTA writes an FP64 partial tile and a
 // reduction kernel sums the splits into C0/C1, mirroring the blocks of a Hermitian product that
 // no tile computed.  Every mbarrier wait is bounded (%globaltimer): on expiry the CTA records an
 // error, leaves its loops, waits for its own copies and MMAs and frees its TMEM.
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
+#include "packed.cuh"
 #include "split_sum.cuh"
 #include "tma.cuh"
 
@@ -36,17 +47,26 @@ namespace {
 constexpr int WB = 64;                    // orbitals per A block and per B half
 constexpr int WN = 2 * WB;                // MMA N
 constexpr int WK = 32;                    // floats of K per stage (one 128-byte swizzled row)
-constexpr int W_THREADS = 576;
-constexpr int W_CVT = 512;                // converter/readout threads
-constexpr int W_MAX_STAGES = 6;
+constexpr int W_CVT = 128;                // threads of one converter warpgroup
+constexpr int W_RO = 256;                 // readout threads
+constexpr int W_THREADS = 128 + 2 * W_CVT + W_RO;
 constexpr uint32_t ROWS = 64 * 128;       // 64 rows of one 128-byte stage row
-// stage layout: [raw A | i*A] [half 0 | half 1] (MMA "hi" operands), then in 3-product mode
-// [A lo | i*A lo] [half 0 lo | half 1 lo]
-constexpr uint32_t STAGE_HI = 4 * ROWS;   // 32 KB
-constexpr uint32_t STAGE_SPLIT = 8 * ROWS;  // 64 KB
-constexpr uint32_t RING = 6 * STAGE_HI;   // 192 KB: 6 single-product or 3 three-product stages
-constexpr uint32_t OFF_BAR = RING;
-constexpr uint32_t SMEM_BYTES = OFF_BAR + 512 + 1024;
+// shared memory: a ring of raw stages [A][half 0 | half 1] (the raw B is the "hi" operand) and one of
+// [half 0 lo | half 1 lo]
+constexpr int RAW = 6, LO = 4;
+constexpr uint32_t RAW_BYTES = 3 * ROWS, LO_BYTES = 2 * ROWS;
+constexpr uint32_t OFF_LO = RAW * RAW_BYTES;
+constexpr uint32_t OFF_BAR = OFF_LO + LO * LO_BYTES;
+constexpr uint32_t SMEM_BYTES = OFF_BAR + 256 + 1024;
+// TMEM columns: two accumulators, then a ring of LO converted A stages (hi and lo)
+constexpr int A_COL0 = 2 * WN;
+constexpr int TMEM_COLS = 512;
+static_assert(A_COL0 + LO * 2 * WK <= TMEM_COLS, "TMEM columns");
+constexpr int AHEAD = 2;                  // stages of its own that a converter warpgroup has in flight
+static_assert(RAW == 2 * AHEAD + 2 && LO == 4, "the slots that the stage two back frees");
+// registers a thread: 640 threads start with 96; MMA 24, converters 48, readout 176 (472 of 480 a lane of each group)
+constexpr int R_MMA = 24, R_CVT = 48, R_RO = 176;
+static_assert(R_MMA + 2 * R_CVT + 2 * R_RO <= 5 * 96, "register split");
 constexpr uint64_t TIMEOUT_NS = 2000000000ull;
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
@@ -67,11 +87,12 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t addr) {
 // instruction descriptor: D f32, A/B tf32, both K-major, N = 128, M = 128
 constexpr uint32_t IDESC_W = (1u << 4) | (2u << 7) | (2u << 10) | (uint32_t(WN >> 3) << 17) | (uint32_t(128 >> 4) << 24);
 
-__device__ __forceinline__ void mma_w(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+// A from TMEM (128 lanes by 8 columns), B from shared memory
+__device__ __forceinline__ void mma_w(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t accumulate) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(IDESC_W), "r"(accumulate)
+      " tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "r"(tmem_a), "l"(bdesc), "r"(IDESC_W), "r"(accumulate)
       : "memory");
 }
 
@@ -92,6 +113,15 @@ __device__ __forceinline__ void ld8(uint32_t taddr, float (&v)[8]) {
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 8 columns of this warp's TMEM lanes
+__device__ __forceinline__ void st8(uint32_t taddr, float4 a, float4 b) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr),
+               "r"(__float_as_uint(a.x)), "r"(__float_as_uint(a.y)), "r"(__float_as_uint(a.z)), "r"(__float_as_uint(a.w)),
+               "r"(__float_as_uint(b.x)), "r"(__float_as_uint(b.y)), "r"(__float_as_uint(b.z)), "r"(__float_as_uint(b.w))
+               : "memory");
+}
+__device__ __forceinline__ void wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
 __device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
 // 16-byte shared-memory accesses by 32-bit shared-window address
 __device__ __forceinline__ float4 lds128(uint32_t a) {
@@ -102,8 +132,11 @@ __device__ __forceinline__ float4 lds128(uint32_t a) {
 __device__ __forceinline__ void sts128(uint32_t a, float4 v) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
+__device__ __forceinline__ float4 hi4(float4 v) { return make_float4(tf32_hi(v.x), tf32_hi(v.y), tf32_hi(v.z), tf32_hi(v.w)); }
 __device__ __forceinline__ float4 lo4(float4 v) {
-  return make_float4(v.x - tf32_hi(v.x), v.y - tf32_hi(v.y), v.z - tf32_hi(v.z), v.w - tf32_hi(v.w));
+  const c64 a = rl::psub(c64{v.x, v.y}, c64{tf32_hi(v.x), tf32_hi(v.y)});
+  const c64 b = rl::psub(c64{v.z, v.w}, c64{tf32_hi(v.z), tf32_hi(v.w)});
+  return make_float4(a.re, a.im, b.re, b.im);
 }
 __device__ __forceinline__ float4 times_i(float4 v) { return make_float4(-v.y, v.x, -v.w, v.z); }
 
@@ -113,34 +146,56 @@ struct WideTile {
 };
 
 struct WideArgs {
+  const float *A, *B0, *B1;
+  int N1, N2;
+  int row;  // floats of an orbital
   int stages_total;
   int stages_per_split;
   int split3;
   int period;
 };
 
+// 16 bytes from global to shared memory, the bytes from `bytes` on as zeros
+__device__ __forceinline__ void cp16(uint32_t dst, const float* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+// barrier 1 + g of one converter warpgroup; whether every thread brought `ok`
+__device__ __forceinline__ bool group_all(int g, bool ok) {
+  int r;
+  if (g == 0)
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n barrier.cta.red.and.pred q, 1, 128, p;\n selp.s32 %0, 1, 0, q;\n}\n"
+        : "=r"(r)
+        : "r"(int(ok))
+        : "memory");
+  else
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n barrier.cta.red.and.pred q, 2, 128, p;\n selp.s32 %0, 1, 0, q;\n}\n"
+        : "=r"(r)
+        : "r"(int(ok))
+        : "memory");
+  return r != 0;
+}
+
 __global__ void __launch_bounds__(W_THREADS, 1)
-    k_gram_tc_wide(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
-                   const __grid_constant__ CUtensorMap tmB1, const WideTile* __restrict__ tiles, WideArgs P,
-                   double* __restrict__ part, int* __restrict__ err) {
+    k_gram_tc_wide(const WideTile* __restrict__ tiles, WideArgs P, double* __restrict__ part, int* __restrict__ err) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char* sm = smem_raw + (base - raw);
-  const int NS = P.split3 ? 3 : 6;
-  const uint32_t stage_bytes = P.split3 ? STAGE_SPLIT : STAGE_HI;
   const uint32_t bar0 = base + OFF_BAR;
-  auto bar_full = [&](int s) { return bar0 + 8u * s; };
-  auto bar_cvt = [&](int s) { return bar0 + 8u * (W_MAX_STAGES + s); };
-  auto bar_empty = [&](int s) { return bar0 + 8u * (2 * W_MAX_STAGES + s); };
-  auto bar_acc_full = [&](int b) { return bar0 + 8u * (3 * W_MAX_STAGES + b); };
-  auto bar_acc_empty = [&](int b) { return bar0 + 8u * (3 * W_MAX_STAGES + 2 + b); };
-  const uint32_t bar_drain = bar0 + 8u * (3 * W_MAX_STAGES + 4);
-  volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(sm + OFF_BAR + 256);
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(sm + OFF_BAR + 264);
-  auto stg = [&](int s) { return base + uint32_t(s) * stage_bytes; };
+  auto bar_cvt = [&](int it) { return bar0 + 8u * (it % RAW); };
+  auto bar_empty = [&](int it) { return bar0 + 8u * (RAW + it % RAW); };
+  auto bar_acc_full = [&](int b) { return bar0 + 8u * (2 * RAW + b); };
+  auto bar_acc_empty = [&](int b) { return bar0 + 8u * (2 * RAW + 2 + b); };
+  const uint32_t bar_drain = bar0 + 8u * (2 * RAW + 4);
+  volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(sm + OFF_BAR + 192);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(sm + OFF_BAR + 200);
+  auto raw_stage = [&](int it) { return base + uint32_t(it % RAW) * RAW_BYTES; };
+  auto lo_stage = [&](int it) { return base + OFF_LO + uint32_t(it % LO) * LO_BYTES; };
+  auto a_cols = [&](int it) { return uint32_t(A_COL0 + (it % LO) * 2 * WK); };
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, group = tid >> 7;
   const int tile = blockIdx.x, split = blockIdx.y;
   const int st0 = split * P.stages_per_split;
   const int st1 = min(P.stages_total, st0 + P.stages_per_split);
@@ -149,22 +204,21 @@ __global__ void __launch_bounds__(W_THREADS, 1)
   const int nper = (nst + period - 1) / period;
 
   if (tid == 0) {
-    for (int s = 0; s < NS; ++s) {
-      mbar_init(bar_full(s), 1);
+    for (int s = 0; s < RAW; ++s) {
       mbar_init(bar_cvt(s), W_CVT);
       mbar_init(bar_empty(s), 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(bar_acc_full(b), 1);
-      mbar_init(bar_acc_empty(b), W_CVT);
+      mbar_init(bar_acc_empty(b), W_RO);
     }
     mbar_init(bar_drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + OFF_BAR + 256),
-                 "r"(2 * WN)
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + OFF_BAR + 192),
+                 "r"(TMEM_COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -177,157 +231,177 @@ __global__ void __launch_bounds__(W_THREADS, 1)
     *abort_flag = 1;
   };
 
-  if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      const WideTile T = tiles[tile];
-      const CUtensorMap* h0 = T.m0 == 1 ? &tmB1 : &tmB0;
-      // an absent second half re-reads the first (its columns are never reduced)
-      const CUtensorMap* h1 = T.m1 < 0 ? h0 : (T.m1 == 1 ? &tmB1 : &tmB0);
-      const int c1 = T.m1 < 0 ? T.c0 : T.c1;
-      int issued = 0;
+  if (group == 0) {
+    // ---------------- MMA issuer (one lane) ----------------
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R_MMA));
+    if (tid == 0) {
       for (int it = 0; it < nst && !*abort_flag; ++it) {
-        const int s = it % NS;
-        if (it >= NS && !mbar_wait(bar_empty(s), ((it / NS) - 1) & 1, TIMEOUT_NS)) {
-          fail_out(1);
-          break;
-        }
-        mbar_arrive_expect_tx(bar_full(s), 3 * ROWS);
-        const int k = (st0 + it) * WK;
-        tma_load_4d(stg(s), &tmA, k, T.r * WB, 0, 0, bar_full(s));
-        tma_load_4d(stg(s) + 2 * ROWS, h0, k, T.c0 * WB, 0, 0, bar_full(s));
-        tma_load_4d(stg(s) + 3 * ROWS, h1, k, c1 * WB, 0, 0, bar_full(s));
-        issued = it + 1;
-      }
-      // loads still in flight must land before the CTA's shared memory is released
-      for (int it = max(0, issued - NS); it < issued; ++it)
-        if (!mbar_wait(bar_full(it % NS), (it / NS) & 1, TIMEOUT_NS)) atomicOr(err, 128);
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      for (int it = 0; it < nst && !*abort_flag; ++it) {
-        const int s = it % NS;
         const int per = it / period, b = per & 1;
         if (it % period == 0 && per >= 2 && !mbar_wait(bar_acc_empty(b), ((per / 2) - 1) & 1, TIMEOUT_NS)) {
           fail_out(2);
           break;
         }
-        if (!mbar_wait(bar_cvt(s), (it / NS) & 1, TIMEOUT_NS)) {
+        if (!mbar_wait(bar_cvt(it), (it / RAW) & 1, TIMEOUT_NS)) {
           fail_out(4);
           break;
         }
         fence_after();
         const uint32_t d = tmem + uint32_t(b * WN);
-        const uint32_t ahi = stg(s), bhi = stg(s) + 2 * ROWS;
-        const uint32_t alo = stg(s) + 4 * ROWS, blo = stg(s) + 6 * ROWS;
+        const uint32_t ahi = tmem + a_cols(it), alo = ahi + WK;
+        const uint32_t bhi = raw_stage(it) + ROWS, blo = lo_stage(it);
 #pragma unroll
         for (int kk = 0; kk < WK / 8; ++kk) {
           const uint32_t off = uint32_t(kk * 32);
           const uint32_t first = (it % period == 0 && kk == 0) ? 0u : 1u;
-          mma_w(d, desc_sw128(ahi + off), desc_sw128(bhi + off), first);
+          mma_w(d, ahi + 8 * kk, desc_sw128(bhi + off), first);
           if (P.split3) {
-            mma_w(d, desc_sw128(ahi + off), desc_sw128(blo + off), 1u);
-            mma_w(d, desc_sw128(alo + off), desc_sw128(bhi + off), 1u);
+            mma_w(d, ahi + 8 * kk, desc_sw128(blo + off), 1u);
+            mma_w(d, alo + 8 * kk, desc_sw128(bhi + off), 1u);
           }
         }
-        commit_w(bar_empty(s));
+        commit_w(bar_empty(it));
         if (it % period == period - 1 || it == nst - 1) commit_w(bar_acc_full(b));
       }
       // all issued MMAs complete before TMEM is freed
       commit_w(bar_drain);
       if (!mbar_wait(bar_drain, 0, TIMEOUT_NS)) atomicOr(err, 256);
     }
-  } else {
-    // ---------------- converters + readout (warps 2..17) ----------------
-    const int ct = tid - 64;          // 0..511
-    const int wg = (warp - 2) >> 2;   // accumulator columns [32 wg, 32 wg + 32)
-    const int quad = warp & 3;        // TMEM lane quarter
-    const uint32_t lane_base = uint32_t(32 * quad) << 16;
-    float sum[32], comp[32];
+    __syncwarp();
+  } else if (group <= 2) {
+    // ---------------- converters: warpgroup g takes the stages of its parity ----------------
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R_CVT));
+    const int g = group - 1, ct = tid & 127;
+    const WideTile T = tiles[tile];
+    // copies: chunk ct & 7 (16 bytes) of the rows (ct >> 3) + 16 j of A (j < 4) and of the halves (4 each); a row's
+    // chunks are swizzled by its index mod 8, which is that of ct >> 3
+    const int crow = ct >> 3;
+    const uint32_t cdst = uint32_t(crow) * 128u + uint32_t((ct & 7) ^ (crow & 7)) * 16u;
+    const size_t row16 = size_t(16) * P.row;
+    const int ra = T.r * WB + crow, rb = T.c0 * WB + crow;
+    // Rows past a matrix, and an absent second half, are not copied: whatever their shared memory holds reaches only
+    // accumulator entries that are never reduced.
+    const bool two = T.m1 >= 0;
+    const int rc = two ? T.c1 * WB + crow : P.N2;
+    const float* const pb = T.m0 == 1 ? P.B1 : P.B0;
+    const float* const pc = T.m1 == 1 ? P.B1 : P.B0;
+    const int na = (P.N1 - ra + 15) / 16, nb = (P.N2 - rb + 15) / 16, nc = (P.N2 - rc + 15) / 16;
+    const int kc = 4 * (ct & 7);
+    const float* const qa = P.A + size_t(ra) * P.row + kc;
+    const float* const qb = pb + size_t(rb) * P.row + kc;
+    const float* const qc = pc + size_t(rc) * P.row + kc;
+    auto copy = [&](int it) {
+      const uint32_t dst = raw_stage(it) + cdst;
+      const int k = (st0 + it) * WK;
+      // a row's end: a chunk is in it whole or not at all (rows are a multiple of four floats), zeros in its place
+      const int bytes = k + kc < P.row ? 16 : 0;
+      const int kin = bytes ? k : -kc;
+      auto rows4 = [&](const float* q, int n, uint32_t d) {
 #pragma unroll
-    for (int c = 0; c < 32; ++c) sum[c] = comp[c] = 0.f;
-    int readouts = 0;
+        for (int j = 0; j < 4; ++j, q += row16)
+          if (j < n) cp16(d + uint32_t(j) * 2048u, q, bytes);
+      };
+      rows4(qa + kin, na, dst);
+      rows4(qb + kin, nb, dst + ROWS);
+      rows4(qc + kin, nc, dst + 2 * ROWS);
+    };
+    auto commit_copies = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+    for (int n = 0; n < AHEAD; ++n) {
+      if (g + 2 * n < nst) copy(g + 2 * n);
+      commit_copies();
+    }
+    // A: this thread's TMEM lane ct is row ct of the MMA's A: orbital row ct & 63, times i from 64 on
+    const int arow = ct & (WB - 1), sw = arow & 7;
+    const bool imag = ct >= WB;
+    const uint32_t lane_base = uint32_t(32 * (warp & 3)) << 16;
+    for (int it = g; it < nst; it += 2) {
+      const bool ok = *abort_flag == 0;
+      asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD - 1) : "memory");
+      if (!group_all(g, ok)) break;  // every thread's copies of the stage are there
+      fence_after();
+      const uint32_t st = raw_stage(it);
+      const uint32_t at = tmem + lane_base + a_cols(it);
+      const uint32_t ast = st + uint32_t(arow) * 128u;
+      auto rows_a = [&](auto turn) {
+#pragma unroll
+        for (int c = 0; c < 8; c += 2) {
+          const float4 r0 = lds128(ast + uint32_t(c ^ sw) * 16u), r1 = lds128(ast + uint32_t((c + 1) ^ sw) * 16u);
+          const float4 a0 = turn ? times_i(r0) : r0, a1 = turn ? times_i(r1) : r1;
+          st8(at + 4 * c, hi4(a0), hi4(a1));
+          if (P.split3) st8(at + WK + 4 * c, lo4(a0), lo4(a1));
+        }
+      };
+      if (imag)
+        rows_a(std::true_type{});
+      else
+        rows_a(std::false_type{});
+      if (P.split3) {
+        // a lo chunk has the swizzled position of its raw one
+        const uint32_t src = st + ROWS + uint32_t(ct) * 16u, dst = lo_stage(it) + uint32_t(ct) * 16u;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) sts128(dst + 2048u * j, lo4(lds128(src + 2048u * j)));
+      }
+      wait_st();
+      fence_before();
+      fence_proxy_async_smem();
+      mbar_arrive(bar_cvt(it));
+      // once the stage two back is multiplied its raw slot takes the copy for it + 2 AHEAD (RAW = 2 AHEAD + 2), and its
+      // slots in shared memory and TMEM (LO = 4) the next conversion
+      if (it >= 2 && !mbar_wait(bar_empty(it - 2), ((it - 2) / RAW) & 1, TIMEOUT_NS)) fail_out(16);
+      if (it + 2 * AHEAD < nst) copy(it + 2 * AHEAD);
+      commit_copies();
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+  } else {
+    // ---------------- readout: warpgroup h owns the accumulator columns [64 h, 64 h + 64) ----------------
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R_RO));
+    const int h = group - 3, quad = warp & 3;
+    const uint32_t lane_base = uint32_t(32 * quad) << 16;
+    c64 sum[32], comp[32];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) sum[c] = comp[c] = c64{0.f, 0.f};
     // waits and aborts are decided per warp (vote), so the .sync.aligned TMEM loads run converged
-    auto readout = [&](int per) -> bool {
+    for (int per = 0; per < nper; ++per) {
       const int b = per & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(bar_acc_full(b), (per / 2) & 1, TIMEOUT_NS))) return false;
+      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(bar_acc_full(b), (per / 2) & 1, TIMEOUT_NS))) {
+        fail_out(32);
+        break;
+      }
       fence_after();
 #pragma unroll
-      for (int c0 = 0; c0 < 32; c0 += 8) {
+      for (int c0 = 0; c0 < 64; c0 += 8) {
         float v[8];
-        ld8(tmem + lane_base + uint32_t(b * WN + 32 * wg + c0), v);
+        ld8(tmem + lane_base + uint32_t(b * WN + 64 * h + c0), v);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float y = v[i] - comp[c0 + i];
-          const float t = sum[c0 + i] + y;
-          comp[c0 + i] = (t - sum[c0 + i]) - y;
-          sum[c0 + i] = t;
+        for (int i = 0; i < 4; ++i) {
+          const int c = c0 / 2 + i;
+          const c64 y = rl::psub(c64{v[2 * i], v[2 * i + 1]}, comp[c]);
+          const c64 t = rl::padd(sum[c], y);
+          comp[c] = rl::psub(rl::psub(t, sum[c]), y);
+          sum[c] = t;
+          // added up before the next columns are loaded: eight loads in flight would hold 64 registers
+          asm volatile("" : "+f"(sum[c].re), "+f"(sum[c].im), "+f"(comp[c].re), "+f"(comp[c].im)::"memory");
         }
       }
       fence_before();
       mbar_arrive(bar_acc_empty(b));
-      return true;
-    };
-    // chunk ct of the A block (64 rows x 8 chunks of 16 bytes) and chunks ct, ct + 512 of the
-    // B halves (128 rows); a warp's 32 chunks are 512 contiguous bytes.  Rows r and r + 64 share
-    // the swizzle phase (r & 7), so a chunk is written at the same position of the other row.
-    const uint32_t offa = uint32_t(ct >> 3) * 128u + uint32_t(ct & 7) * 16u;
-    const uint32_t offb0 = offa, offb1 = offa + 64u * 128u;
-    constexpr int LAG = 2;  // read a period out once the converters are LAG stages past its end
-    for (int it = 0; it < nst; ++it) {
-      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
-      const int s = it % NS;
-      if (!__all_sync(0xffffffffu, mbar_wait(bar_full(s), (it / NS) & 1, TIMEOUT_NS))) {
-        fail_out(8);
-        break;
-      }
-      const uint32_t st = stg(s);
-      {
-        const float4 a = lds128(st + offa);
-        sts128(st + ROWS + offa, times_i(a));
-        if (P.split3) {
-          const float4 al = lo4(a);
-          sts128(st + 4 * ROWS + offa, al);
-          sts128(st + 5 * ROWS + offa, times_i(al));
-        }
-      }
-      if (P.split3) {
-        sts128(st + 6 * ROWS + offb0, lo4(lds128(st + 2 * ROWS + offb0)));
-        sts128(st + 6 * ROWS + offb1, lo4(lds128(st + 2 * ROWS + offb1)));
-      }
-      fence_proxy_async_smem();
-      mbar_arrive(bar_cvt(s));
-      const int lagged = it - LAG;
-      if (lagged >= 0 && (lagged % period == period - 1)) {
-        if (!readout(lagged / period)) {
-          fail_out(32);
-          break;
-        }
-        ++readouts;
-      }
-    }
-    while (readouts < nper) {
-      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
-      if (!readout(readouts)) {
-        fail_out(64);
-        break;
-      }
-      ++readouts;
     }
     // FP64 partial: rows 0..63 real part, 64..127 imaginary part; columns 0..63 half 0, 64..127 half 1
     const int row = 32 * quad + lane;
-    double* out = part + ((size_t(split) * gridDim.x + tile) * 128 + row) * WN + 32 * wg;
+    double* out = part + ((size_t(split) * gridDim.x + tile) * 128 + row) * WN + 64 * h;
 #pragma unroll
-    for (int c = 0; c < 32; ++c) out[c] = double(sum[c]) - double(comp[c]);
+    for (int c = 0; c < 32; ++c) {
+      const double2 v = make_double2(double(sum[c].re) - double(comp[c].re), double(sum[c].im) - double(comp[c].im));
+      asm volatile("st.global.v2.f64 [%0], {%1, %2};" ::"l"(out + 2 * c), "d"(v.x), "d"(v.y) : "memory");
+    }
   }
   // teardown: every role has left its loop; free TMEM
   fence_before();
   __syncthreads();
-  if (warp == 1) {
+  if (warp == 0) {
     __syncwarp();
     fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * WN) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
   }
 }
 
@@ -440,17 +514,17 @@ void gram_tc_wide(pt_ctx* ctx, const c64* A, const c64* B0, c128* C0, const c64*
   once([] {
     PT_CUDA_CHECK(cudaFuncSetAttribute(k_gram_tc_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
   });
-  CUtensorMap ta, tb0, tb1;
-  const uint64_t da[4] = {2 * ng, uint64_t(N1), 1, 1}, db[4] = {2 * ng, uint64_t(N2), 1, 1};
-  const uint64_t sa[3] = {2 * ng * 4, 2 * ng * 4 * uint64_t(N1), 2 * ng * 4 * uint64_t(N1)};
-  const uint64_t sb[3] = {2 * ng * 4, 2 * ng * 4 * uint64_t(N2), 2 * ng * 4 * uint64_t(N2)};
-  const uint32_t box[4] = {WK, WB, 1, 1};
-  encode_tmap_4d_f32(&ta, A, da, sa, box, CU_TENSOR_MAP_SWIZZLE_128B);
-  encode_tmap_4d_f32(&tb0, B0, db, sb, box, CU_TENSOR_MAP_SWIZZLE_128B);
-  encode_tmap_4d_f32(&tb1, two ? B1 : B0, db, sb, box, CU_TENSOR_MAP_SWIZZLE_128B);
-  WideArgs P{stages_total, sps, split3 ? 1 : 0, std::max(1, ctx->tc_period)};
-  PT_LAUNCH(k_gram_tc_wide, dim3(pl->ntiles, splits), W_THREADS, SMEM_BYTES, st, ta, tb0, tb1, pl->tiles, P, part,
-            err);
+  WideArgs P{reinterpret_cast<const float*>(A),
+             reinterpret_cast<const float*>(B0),
+             reinterpret_cast<const float*>(two ? B1 : B0),
+             N1,
+             N2,
+             int(2 * ng),
+             stages_total,
+             sps,
+             split3 ? 1 : 0,
+             std::max(1, ctx->tc_period)};
+  PT_LAUNCH(k_gram_tc_wide, dim3(pl->ntiles, splits), W_THREADS, SMEM_BYTES, st, pl->tiles, P, part, err);
   const size_t n = size_t(N1) * N2;
   const int nbi = (N1 + WB - 1) / WB, nbj = (N2 + WB - 1) / WB;
   PT_LAUNCH_SPLIT_SUM(k_gram_tc_wide_reduce, n, two ? 2u : 1u, splits, st, part, splits, pl->ntiles, pl->lut, nbi, nbj, N1,
