@@ -11,9 +11,8 @@
 //
 // The orbitals are stored orbital-major (r contiguous for each k), the transpose of the K-major
 // operand the tensor core reads, so TMA brings in a [16 orbitals][128 points] block of complex64
-// values and a converter warpgroup writes it out as 128 K-major rows of 32 floats (128B swizzle),
-// once as the raw values (the tensor core reads their TF32 bits: "hi") and once as the FP32
-// remainders x - tf32(x) ("lo").  B' is written once per call as the shared-memory images of
+// values and a converter warpgroup writes it to TMEM, a lane of 32 floats per point, once as their
+// TF32 parts ("hi") and once as the FP32 remainders x - tf32(x) ("lo"): the MMA's A operand.  B' is written once per call as the shared-memory images of
 // its stages (for every 128-row block and 32-float K stage, the hi and the lo tile in the 128B
 // swizzle the tensor core reads, 32 KB contiguous), so a stage's B operands arrive with one bulk
 // copy instead of a tiled load of 2 x 128 rows of 128 bytes.  Products summed per tile:
@@ -22,18 +21,20 @@
 // Warp roles (448 threads): warp 0 TMA producer, warp 1 TMEM allocation and MMA issue (one
 // lane), warps 2..5 converter, warps 6..9 and 10..13 TMEM readout and epilogue of half of the columns each
 // (alpha is folded into B'; the epilogue adds the extra terms and stores complex64).  B' stages have a
-// ring of their own, three deep, so that their 32 KB copies run ahead of the conversions (with one ring of
-// two for both operands a stage's buffers took the MMAs, the copy and the conversion in turn; 54^3, 200 x 200
-// 512 -> 446 us, 60^3, 150 x 150 434 -> 366, 64^3, 320 x 320 1371 -> 1275).  What bounds it now is shared
-// memory: by count 96 KB of operand reads and 96 KB of copies and conversions a stage, 1500 cycles; two
-// converter warpgroups (96 registers a thread) ran slower, 507 us.  CTAs are persistent and walk
-// the tiles with a grid stride; the two TMEM accumulators alternate between periods, so the
+// ring of their own, so that their 32 KB copies run ahead of the conversions (with one ring of two for both
+// operands a stage's buffers took the MMAs, the copy and the conversion in turn; 54^3, 200 x 200 512 -> 446 us, 60^3,
+// 150 x 150 434 -> 361, 64^3, 320 x 320 1371 -> 1266), and A operands in TMEM in place of swizzled rows in shared memory
+// take a third off the traffic of its pipe (446 -> 419, 361 -> 345, 1266 -> 1198).  What bounds it now are the 48 KB of
+// operands that a CTA takes in for each stage, at 48 GB/s (7.3 TB/s in all).  Two converter warpgroups at 96
+// registers a thread ran slower (507 us).
+//   CTAs are persistent and walk the tiles with a grid stride; the two TMEM accumulators alternate between periods, so the
 // epilogue of one tile overlaps the MMAs of the next.  Every wait is bounded (%globaltimer); on
 // expiry the CTA records an error, leaves its loops, drains its own copies and tensor-core work
 // and frees its TMEM.
 #include <algorithm>
 
 #include "internal.h"
+#include "packed.cuh"
 #include "tma.cuh"
 
 namespace pt {
@@ -44,19 +45,21 @@ constexpr int RM = 128;                 // grid points per tile (MMA M)
 constexpr int RJ = 64;                  // output orbitals per tile (MMA N = 2 RJ real columns)
 constexpr int NC = 2 * RJ;              // 128 real output columns
 constexpr int KO = 16;                  // orbitals per K stage (32 floats of K')
-constexpr int RA = 3;                   // raw A stages
-constexpr int RC = 2;                   // converted A stages
-constexpr int RB = 3;                   // B stages
+constexpr int RA = 5;                   // raw A stages
+constexpr int RC = 4;                   // converted A stages, in TMEM
+constexpr int RB = 4;                   // B stages
 constexpr int RO = 2;                   // readout warpgroups (NC / RO columns each)
 constexpr int THREADS = 64 + 128 * (1 + RO);
 constexpr uint32_t RAW_BYTES = KO * RM * 8;          // 16 KB: [16 orbitals][128 points] complex64
 constexpr uint32_t OP_BYTES = 128 * 128;             // 16 KB: 128 rows x 32 floats, swizzled
-constexpr uint32_t CST_BYTES = 2 * OP_BYTES;         // A hi | A lo, or B hi | B lo
-constexpr uint32_t OFF_C = 0;                        // converted ring (1024-aligned stages)
-constexpr uint32_t OFF_B = RC * CST_BYTES;           // B ring
-constexpr uint32_t OFF_RAW = OFF_B + RB * CST_BYTES;
+constexpr uint32_t CST_BYTES = 2 * OP_BYTES;         // B hi | B lo
+constexpr uint32_t OFF_RAW = RB * CST_BYTES;         // after the B ring (1024-aligned stages)
 constexpr uint32_t OFF_BAR = OFF_RAW + RA * RAW_BYTES;  // 212992
-constexpr uint32_t SMEM_BYTES = OFF_BAR + 256 + 1024;
+constexpr uint32_t SMEM_BYTES = OFF_BAR + 512 + 1024;
+// TMEM columns: two accumulators, then RC converted A stages (hi and lo)
+constexpr int A_COL0 = 2 * NC, A_COLS = 4 * KO;
+constexpr int TMEM_COLS = 512;
+static_assert(A_COL0 + RC * A_COLS <= TMEM_COLS, "TMEM columns");
 constexpr uint64_t TIMEOUT_NS = 2000000000ull;
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
@@ -77,11 +80,12 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
 // instruction descriptor: D f32, A/B tf32, K-major both, N = NC, M = RM
 constexpr uint32_t IDESC = (1u << 4) | (2u << 7) | (2u << 10) | (uint32_t(NC >> 3) << 17) | (uint32_t(RM >> 4) << 24);
 
-__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+// A from TMEM (128 lanes by 8 columns), B from shared memory
+__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t accumulate) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(IDESC), "r"(accumulate)
+      " tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "r"(tmem_a), "l"(bdesc), "r"(IDESC), "r"(accumulate)
       : "memory");
 }
 
@@ -104,6 +108,16 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+
+// 8 columns of this warp's TMEM lanes
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&v)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr),
+               "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
+               "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
+               "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7]))
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
 
@@ -168,13 +182,12 @@ __global__ void __launch_bounds__(THREADS, 1)
   auto bar_acc_full = [&](int b) { return bar0 + 8u * (NB + 2 * RC + b); };
   auto bar_acc_empty = [&](int b) { return bar0 + 8u * (NB + 2 * RC + 2 + b); };
   const uint32_t bar_drain = bar0 + 8u * (NB + 2 * RC + 4);
-  static_assert(8 * (NB + 2 * RC + 5) <= 192, "barriers below the TMEM address");
-  volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(sm + OFF_BAR + 192);
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(sm + OFF_BAR + 200);
+  static_assert(8 * (NB + 2 * RC + 5) <= 256, "barriers below the TMEM address");
+  volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(sm + OFF_BAR + 256);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(sm + OFF_BAR + 264);
   auto a_raw = [&](int s) { return base + OFF_RAW + uint32_t(s) * RAW_BYTES; };
-  auto c_ahi = [&](int s) { return base + OFF_C + uint32_t(s) * CST_BYTES; };
-  auto c_alo = [&](int s) { return c_ahi(s) + OP_BYTES; };
-  auto c_bhi = [&](int s) { return base + OFF_B + uint32_t(s) * CST_BYTES; };
+  auto c_a = [&](int s) { return uint32_t(A_COL0 + s * A_COLS); };  // TMEM column of a converted stage
+  auto c_bhi = [&](int s) { return base + uint32_t(s) * CST_BYTES; };
   auto c_blo = [&](int s) { return c_bhi(s) + OP_BYTES; };
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -206,8 +219,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     fence_mbar_init();
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + OFF_BAR + 192),
-                 "r"(2 * NC)
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + OFF_BAR + 256),
+                 "r"(TMEM_COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -274,14 +287,15 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         tc_fence_after();
         const uint32_t d = tmem + uint32_t(b * NC);
+        const uint32_t ahi = tmem + c_a(sc), alo = ahi + 2 * KO;
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
           const uint32_t off = uint32_t(kk * 32);
           const uint32_t acc = (first && kk == 0) ? 0u : 1u;
-          mma_tf32(d, smem_desc_sw128(c_ahi(sc) + off), smem_desc_sw128(c_bhi(sb) + off), acc);
+          mma_tf32(d, ahi + 8 * kk, smem_desc_sw128(c_bhi(sb) + off), acc);
           if (P.split3) {
-            mma_tf32(d, smem_desc_sw128(c_ahi(sc) + off), smem_desc_sw128(c_blo(sb) + off), 1u);
-            mma_tf32(d, smem_desc_sw128(c_alo(sc) + off), smem_desc_sw128(c_bhi(sb) + off), 1u);
+            mma_tf32(d, ahi + 8 * kk, smem_desc_sw128(c_blo(sb) + off), 1u);
+            mma_tf32(d, alo + 8 * kk, smem_desc_sw128(c_bhi(sb) + off), 1u);
           }
         }
         mma_commit(bar_c_empty(sc));
@@ -295,8 +309,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (!mbar_wait(bar_drain, 0, TIMEOUT_NS)) atomicOr(err, 256);
     }
   } else if (warp < 6) {
-    // ---------------- converter: raw [16][128] complex64 -> K-major swizzled rows ----------------
-    const int row = tid - 64;  // 0..127: grid point within the tile
+    // ---------------- converter: raw [16][128] complex64 -> a TMEM lane of 32 floats per point ----------------
+    const int row = 32 * (warp & 3) + lane;  // this thread's TMEM lane: grid point within the tile
+    const uint32_t lane_base = uint32_t(32 * (warp & 3)) << 16;
     for (int q = 0; q < nq; ++q) {
       if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
       const int sa = q % RA, sc = q % RC;
@@ -314,18 +329,30 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
       for (int k = 0; k < KO; ++k) v[k] = src[k * RM + row];
       mbar_arrive(bar_a_empty(sa));
-      unsigned char* hi = sm + (c_ahi(sc) - base) + row * 128;
-      unsigned char* lo = sm + (c_alo(sc) - base) + row * 128;
+      tc_fence_after();
+      const uint32_t at = tmem + lane_base + c_a(sc);
 #pragma unroll
-      for (int ch = 0; ch < 8; ++ch) {
-        const uint32_t pos = uint32_t((ch ^ (row & 7)) * 16);
-        const float4 h = make_float4(v[2 * ch].x, v[2 * ch].y, v[2 * ch + 1].x, v[2 * ch + 1].y);
-        *reinterpret_cast<float4*>(hi + pos) = h;
-        if (P.split3)
-          *reinterpret_cast<float4*>(lo + pos) =
-              make_float4(h.x - tf32_hi(h.x), h.y - tf32_hi(h.y), h.z - tf32_hi(h.z), h.w - tf32_hi(h.w));
+      for (int k = 0; k < KO; k += 4) {
+        float h[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          h[2 * i] = tf32_hi(v[k + i].x);
+          h[2 * i + 1] = tf32_hi(v[k + i].y);
+        }
+        tmem_st8(at + 2 * k, h);
+        if (P.split3) {
+          float l[8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const c64 d = rl::psub(c64{v[k + i].x, v[k + i].y}, c64{h[2 * i], h[2 * i + 1]});
+            l[2 * i] = d.re;
+            l[2 * i + 1] = d.im;
+          }
+          tmem_st8(at + 2 * KO + 2 * k, l);
+        }
       }
-      fence_proxy_async_smem();
+      tmem_wait_st();
+      tc_fence_before();
       mbar_arrive(bar_c_full(sc));
     }
   } else {
@@ -408,7 +435,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * NC) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
   }
 }
 
