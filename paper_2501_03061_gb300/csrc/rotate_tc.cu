@@ -12,7 +12,8 @@
 // The orbitals are stored orbital-major (r contiguous for each k), the transpose of the K-major
 // operand the tensor core reads, so TMA brings in a [16 orbitals][128 points] block of complex64
 // values and a converter warpgroup writes it to TMEM, a lane of 32 floats per point, once as their
-// TF32 parts ("hi") and once as the FP32 remainders x - tf32(x) ("lo"): the MMA's A operand.  B' is written once per call as the shared-memory images of
+// TF32 parts ("hi") and once as the FP32 remainders x - tf32(x) ("lo"): the MMA's A operand.
+// B' is written once per call as the shared-memory images of
 // its stages (for every 128-row block and 32-float K stage, the hi and the lo tile in the 128B
 // swizzle the tensor core reads, 32 KB contiguous), so a stage's B operands arrive with one bulk
 // copy instead of a tiled load of 2 x 128 rows of 128 bytes.  Products summed per tile:
@@ -24,9 +25,10 @@
 // ring of their own, so that their 32 KB copies run ahead of the conversions (with one ring of two for both
 // operands a stage's buffers took the MMAs, the copy and the conversion in turn; 54^3, 200 x 200 512 -> 446 us, 60^3,
 // 150 x 150 434 -> 361, 64^3, 320 x 320 1371 -> 1266), and A operands in TMEM in place of swizzled rows in shared memory
-// take a third off the traffic of its pipe (446 -> 419, 361 -> 345, 1266 -> 1198).  What bounds it now are the 48 KB of
-// operands that a CTA takes in for each stage, at 48 GB/s (7.3 TB/s in all).  Two converter warpgroups at 96
-// registers a thread ran slower (507 us).
+// take a third off the traffic of its pipe (446 -> 419, 361 -> 345, 1266 -> 1198).  A stage takes about 1900 cycles, of
+// which the MMAs are 770; 48 KB of operands come in for each at 48 GB/s a CTA.  Two converter warpgroups at 96
+// registers a thread ran slower (507 us), and so did two row tiles that share the B' stages (501): the
+// epilogue of both at once leaves the MMAs without a free accumulator, it seems, for longer than the loads saved.
 //   CTAs are persistent and walk the tiles with a grid stride; the two TMEM accumulators alternate between periods, so the
 // epilogue of one tile overlaps the MMAs of the next.  Every wait is bounded (%globaltimer); on
 // expiry the CTA records an error, leaves its loops, drains its own copies and tensor-core work
