@@ -32,11 +32,10 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "Vx·Ψ pair-FFTs/s and PT-IM steps/s vs plain FP64 GPU form; serve p50/p99"
-# DRAM bytes (read + write) per steady-state launch of the 64^3 FP32 exchange kernel: mean of two
-# launches (2.849 and 2.951 GB) of an ncu --set full capture with the 16 x 16 pair tiles the
-# benchmark cell uses (N = 64 orbitals, the same launch shape), taken on the kernel with one 5-D
-# TMA copy per plane or slab; the kernel is unchanged since that capture
-EXCHANGE64_TRAFFIC_PER_LAUNCH = 2.90e9
+# DRAM bytes (read + write) per launch of the 64^3 FP32 exchange kernels, the mean over the 630 launches of an N = 320
+# application: three passes (659, 1013 and 749 MB) for each of 190 tiles of 16 x 16 pairs, and 1147 MB for the three of
+# each of the 20 diagonal tiles, from an ncu capture of the same tiles at N = 64
+EXCHANGE64_TRAFFIC_PER_LAUNCH = 7.67e8
 UNIT = "PT-IM steps/s"
 WORKLOAD = "ptim_ace_step_64^3_N320_128site_L20.5"
 # iteration counts of one benchmark step as the GPU step measured them (ACE builds, inner iterations
@@ -77,7 +76,7 @@ def parse():
     ap.add_argument("--inner-cap", type=float, default=None,
                     help="loosest inner tolerance of the PT-IM step (context option ptim_inner_cap)")
     ap.add_argument("--engine", type=int, default=None, choices=[0, 1, 2, 3],
-                    help="64^3 FP32 exchange engine: 0 launch-pipelined TMA kernel, 1 compile-time tile kernels, "
+                    help="64^3 FP32 exchange engine: 0 whole lines in registers, 1 compile-time tile kernels, "
                          "2 persistent cooperative kernel, 3 pipelined TMA kernel with the fused CD role "
                          "(default: the library's)")
     ap.add_argument("--x64p", type=str, default=None, help="tile,ring,lag of the persistent 64^3 engine")
@@ -1114,7 +1113,7 @@ def run_gb300(args):
                          "algorithmic_bytes_per_launch": alg_per_launch,
                          "traffic_over_algorithmic": (traffic / alg_per_launch) if traffic else None,
                          "launches_per_application": ex_launches_per_app,
-                         "kernel": "pair-FFT exchange (plane/column/plane passes)",
+                         "kernel": "pair-FFT exchange (z lines, planes, z lines and accumulate)",
                          "model": "4 complex fields of Ng per pair FFT (read phit_i, read phi_j, read and write "
                                   "W_j; a symmetric pair FFT counts once)",
                          "frac_six_field_model": (achieved_sym / peak) if achieved_sym else None,

@@ -15,11 +15,12 @@
 // less than the write and the two reads of v_ij that it saves.
 //
 // What bounds it: registers.  A 64-point line is 128 registers, so an SM holds 12 warps (N <= 32: 20),
-// and the passes run at 30-45% of the issue rate and 45-75% of the L1 rate, waiting on the loads
+// and the passes run at 25-45% of the issue rate, 30-55% of the L1 rate and, at 64^3, 4.2-5.2 TB/s of memory
+// (0.63-0.78 of a copy), waiting on the loads
 // and stores of lines between the transforms.  Measured on GB300, one V_x application, all pairs
 // symmetric (this form against the tile kernels, at 64 against the TMA pipeline it replaced):
 //   24^3 N = 64   0.22 against 0.67 ms      48^3 N = 128   6.7 against 18.0 ms
-//   36^3 N = 96   1.83 against 4.66 ms      64^3 N = 96   11.0 against 14.4 ms
+//   36^3 N = 96   1.69 against 4.66 ms      64^3 N = 96    9.7 against 14.4 ms, N = 320 105.5 against 157.4
 // i.e. 0.007-0.009 ns per pair and grid point against 0.012 (64^3) and 0.020-0.026.
 #include "exchange_lines.cuh"
 #include "fft_fixed.cuh"
