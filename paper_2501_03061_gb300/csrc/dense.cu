@@ -97,7 +97,10 @@ __global__ void __launch_bounds__(ST* ST* SG) k_gemm_small(char opA, char opB, i
 // ---------------------------------------------------------------- Jacobi ----
 // pair partner of position k in round r of the circle method on Np (even) players
 __device__ __forceinline__ void jacobi_pair(int k, int r, int Np, int* p, int* q) {
-  auto idx = [&](int i) { return i == 0 ? 0 : ((i - 1 + r) % (Np - 1)) + 1; };
+  auto idx = [&](int i) {  // 1 + (i - 1 + r) mod (Np - 1), r < Np - 1
+    const int j = i + r;
+    return i == 0 ? 0 : j >= Np ? j - (Np - 1) : j;
+  };
   const int a = idx(k), b = idx(Np - 1 - k);
   *p = min(a, b);
   *q = max(a, b);
@@ -272,9 +275,15 @@ __host__ __device__ inline bool jacobi32_done(double off, double off0, double pr
   return !(off > floor2) || off <= 1e-14 * N * off0 || (off <= 1e-9 * off0 && off > 0.25 * prev);
 }
 
-// One CTA, E and the basis in shared memory (N <= J32_MAX): whole sweeps, two barriers a round (0.7 us at N = 48 against
-// 8.7 us of k_jacobi_round, which is a launch and a chain of FP64 instructions).  X: the basis, as FP64.
+// One CTA, E and the basis in shared memory (N <= J32_MAX): whole sweeps, two barriers a round (under 1 us at N = 48 against
+// 8.7 us of k_jacobi_round, which is a launch and a chain of FP64 instructions).  A thread for each 2 x 2 block of E, as far
+// as a CTA has them, and its place in E and V without divisions in the rounds (N = 48, the two passes of a solve:
+// 580 -> 445 us).  X: the basis, as FP64.
 constexpr int J32_MAX = 96, J32_THREADS = 1024;
+inline int j32_threads(int N) {
+  const int half = (N + 1) / 2;
+  return std::min(J32_THREADS, std::max(64, (half * half + 31) / 32 * 32));
+}
 constexpr size_t j32_smem(int N) { return 2 * size_t(N) * (N | 1) * sizeof(c64); }
 __global__ void __launch_bounds__(J32_THREADS) k_jacobi32_cta(const c128* __restrict__ A, int N, float floor2,
                                                               c128* __restrict__ X) {
@@ -286,8 +295,10 @@ __global__ void __launch_bounds__(J32_THREADS) k_jacobi32_cta(const c128* __rest
   __shared__ short2 pq[J32_MAX / 2];
   __shared__ float2 dg[J32_MAX];
   __shared__ float red[J32_THREADS / 32];
-  const int t = threadIdx.x;
-  for (int e = t; e < N * N; e += J32_THREADS) {
+  const int t = threadIdx.x, TH = blockDim.x;
+  // rows and columns of this thread's first entry, and the step to its next, of a half wide array
+  const int first_k = t / half, first_l = t - first_k * half, step_k = TH / half, step_l = TH - step_k * half;
+  for (int e = t; e < N * N; e += TH) {
     const int i = e / N, j = e - i * N;
     if (i == j) dg[i] = to_pair(A[e].re);
     a[i * P + j] = to_cx<float>(A[e]);
@@ -297,7 +308,7 @@ __global__ void __launch_bounds__(J32_THREADS) k_jacobi32_cta(const c128* __rest
   for (int sweep = 0; sweep < 12; ++sweep) {
     __syncthreads();
     float off = 0.f;
-    for (int e = t; e < N * N; e += J32_THREADS) {
+    for (int e = t; e < N * N; e += TH) {
       const int i = e / N, j = e - i * N;
       const c64 x = a[i * P + j];
       if (i != j) off += x.re * x.re + x.im * x.im;
@@ -306,7 +317,7 @@ __global__ void __launch_bounds__(J32_THREADS) k_jacobi32_cta(const c128* __rest
     if ((t & 31) == 0) red[t >> 5] = off;
     __syncthreads();
     off = 0.f;
-    for (int w = 0; w < J32_THREADS / 32; ++w) off += red[w];
+    for (int w = 0; w < TH / 32; ++w) off += red[w];
     if (sweep == 0) {
       off0 = off;
       thr2 = fmaxf(1e-15f * off0, floor2) / (float(N) * float(N));
@@ -329,8 +340,11 @@ __global__ void __launch_bounds__(J32_THREADS) k_jacobi32_cta(const c128* __rest
         rot[t] = x;
       }
       __syncthreads();
-      for (int e = t; e < half * half; e += J32_THREADS) {
-        const int k = e / half, l = e - k * half;
+      auto next = [&](int& k, int& l) {
+        k += step_k, l += step_l;
+        if (l >= half) l -= half, ++k;
+      };
+      for (int k = first_k, l = first_l; k < half; next(k, l)) {
         const Rot<float> x = rot[k], y = rot[l];
         if (x.s == 0.f && y.s == 0.f) continue;
         const int p1 = pq[k].x, q1 = pq[k].y, p2 = pq[l].x, q2 = pq[l].y;
@@ -347,8 +361,7 @@ __global__ void __launch_bounds__(J32_THREADS) k_jacobi32_cta(const c128* __rest
         if (in1) a[q1 * P + p2] = x10;
         if (in1 && in2) a[q1 * P + q2] = x11;
       }
-      for (int e = t; e < N * half; e += J32_THREADS) {
-        const int row = e / half, l = e - row * half;
+      for (int row = first_k, l = first_l; row < N; next(row, l)) {
         const Rot<float> y = rot[l];
         const int p = pq[l].x, q = pq[l].y;
         if (y.s == 0.f || q >= N) continue;
@@ -359,7 +372,7 @@ __global__ void __launch_bounds__(J32_THREADS) k_jacobi32_cta(const c128* __rest
     }
   }
   __syncthreads();
-  for (int e = t; e < N * N; e += J32_THREADS) {
+  for (int e = t; e < N * N; e += TH) {
     const c64 x = v[(e / N) * P + e % N];
     X[e] = c128{double(x.re), double(x.im)};
   }
@@ -807,7 +820,7 @@ int heev(pt_ctx* ctx, const c128* S, int N, c128* Q, double* d, cudaStream_t st,
         PT_CUDA_CHECK(
             cudaFuncSetAttribute(k_jacobi32_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, int(j32_smem(J32_MAX))));
       });
-      PT_LAUNCH(k_jacobi32_cta, 1, J32_THREADS, j32_smem(N), st, A0, N, float(floor2), X0);
+      PT_LAUNCH(k_jacobi32_cta, 1, j32_threads(N), j32_smem(N), st, A0, N, float(floor2), X0);
     } else {
       // E and V in buffers that are free until the products below
       c64 *e0 = reinterpret_cast<c64*>(G), *e1 = e0 + size_t(N) * N, *v32 = reinterpret_cast<c64*>(X1);
