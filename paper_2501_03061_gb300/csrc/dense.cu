@@ -802,7 +802,7 @@ int heev(pt_ctx* ctx, const c128* S, int N, c128* Q, double* d, cudaStream_t st,
   // Where the caller asks for less than FP64 rounding (rel_tol): FP32 passes on D + E (see k_jacobi32_cta), each basis
   // made unitary in FP64 by two Newton-Schulz steps (X <- X (3 I - X^* X)/2, the error squared each time) and
   // A <- X^* A X in FP64.  Two passes usually meet the tolerance, whose test stays that of the FP64 sweeps below, which
-  // finish the rest.  A pass costs seven FP64 products and its sweeps (N = 48: 2.05 -> 0.80 ms a solve; N = 320, a launch
+  // finish the rest.  A pass costs seven FP64 products and its sweeps (N = 48: 2.05 -> about 0.67 ms a solve; N = 320, a launch
   // per FP32 round: 25 -> 15 ms).
   for (int pass = 0; rel_tol > 0.0 && pass < 3; ++pass) {
     const double before = h[0];
