@@ -167,14 +167,14 @@ __global__ void __launch_bounds__(accum_columns(N, S) * S, accum_min(N, S))
   const int C = CC ? CC : columns;
   const size_t NG = size_t(N) * C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  // the sources' occupations as floats, NaN for one that is exactly empty (its pair fields may be unwritten): one
-  // FP64 conversion per source and CTA, since FP64 instructions issue every 64 cycles on this part
+  // the sources' occupations as floats: one FP64 conversion per source and CTA, since FP64 instructions issue every 64
+  // cycles on this part
   __shared__ float so[MAXB];
   __shared__ uint32_t tm_holder;
   const bool mir = int(blockIdx.x) >= t.nj;  // the target is one of the tile's sources (mirrored contributions)
   const int g = mir ? blockIdx.x - t.nj : blockIdx.x;
   const int ns = mir ? t.nj : t.ni, s0 = mir ? t.j0 : t.i0, tg = (mir ? t.i0 : t.j0) + g;
-  for (int c = threadIdx.x; c < ns; c += OT * S) so[c] = is_zero(occ + s0 + c) ? __int_as_float(0x7fc00000) : float(occ[s0 + c]);
+  for (int c = threadIdx.x; c < ns; c += OT * S) so[c] = float(occ[s0 + c]);
   uint32_t row = 0;  // address of the thread's row in tensor memory
   if constexpr (tmem) {
     if (threadIdx.x < 32) {
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(accum_columns(N, S) * S, accum_min(N, S))
     const int c = g ^ k;
     if (c >= ns) continue;
     const float d = so[c];
-    if (isnan(d)) continue;
+    if (d == 0.f) continue;  // empty: its pair fields may be unwritten (a NaN is not, and belongs to the result)
     const bool cj = mir || (t.diag && c > g);
     const c64* f = vp + size_t(cj ? g * t.nj + c : c * t.nj + g) * NG;
     const c64* w = sp + size_t(c) * NG;
