@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(256) k_chol_diag(cx<T>* __restrict__ A, int N,
     if (tid < 32) {
       if (tid == 0 && k + 1 < bs) {
         const cx<T> c = a[k + 1][k];
-        a[k + 1][k + 1].re -= (c.re * c.re + c.im * c.im) * r;
+        a[k + 1][k + 1].re -= c.re * (c.re * r) + c.im * (c.im * r);  // c squared would leave the range first
         pivot(k + 1);
       }
     } else {
