@@ -556,6 +556,8 @@ __device__ __forceinline__ bool good_pivot(double x) {
   const long long b = __double_as_longlong(x);
   return b > 0 && b < 0x7ff0000000000000ll;
 }
+__device__ __forceinline__ bool is_zero_bits(float x) { return __float_as_int(x) == 0; }
+__device__ __forceinline__ bool is_zero_bits(double x) { return __double_as_longlong(x) == 0; }
 
 // Factor and inverse of a diagonal block as A = U D U^* (U unit lower triangular): step k subtracts column k's outer product
 // from the trailing triangle and column k from the rows of U^{-1} below it; L = U D^{1/2} and L^{-1} = D^{-1/2} U^{-1}
@@ -571,8 +573,8 @@ __global__ void __launch_bounds__(256) k_chol_diag(cx<T>* __restrict__ A, int N,
   // lower triangle (i >= j) listed column by column: entry (j, i) at j*bs - j(j-1)/2 + (i - j), so
   // the trailing triangle of step k (j > k) is one contiguous range, its first entry the next pivot
   __shared__ unsigned short tri[CB * (CB + 1) / 2];
-  __shared__ T rd[CB], rs[CB];  // reciprocals of the pivots and of their square roots
-  __shared__ int bad;
+  // reciprocals of the pivots (zero: the pivot is not positive and finite) and of their square roots
+  __shared__ T rd[CB], rs[CB];
   pdl_wait();  // the previous panel's trailing update
   pdl_launch_dependents();
   if (*info) return;
@@ -586,21 +588,17 @@ __global__ void __launch_bounds__(256) k_chol_diag(cx<T>* __restrict__ A, int N,
   __syncthreads();
   auto pivot = [&](int k) {  // one thread: a[k][k] is final
     const T d = a[k][k].re;
-    if (good_pivot(d)) rd[k] = T(1) / d;
-    else bad = k + 1;
+    rd[k] = good_pivot(d) ? T(1) / d : T(0);
   };
-  if (tid == 0) {
-    bad = 0;
-    pivot(0);
-  }
+  if (tid == 0) pivot(0);
   __syncthreads();
   const int tri_end = bs * (bs + 1) / 2;
   for (int k = 0; k < bs; ++k) {
-    if (bad) {  // uniform: read behind the barrier that followed its writing
-      if (tid == 0) *info = kb + bad;
+    const T r = rd[k];
+    if (is_zero_bits(r)) {  // uniform: written before the barrier behind this step, which writes rd[k + 1] alone
+      if (tid == 0) *info = kb + k + 1;
       return;
     }
-    const T r = rd[k];
     const int first = (k + 1) * bs - (k + 1) * k / 2;
     if (tid < 32) {
       if (tid == 0 && k + 1 < bs) {

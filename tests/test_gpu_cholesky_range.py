@@ -50,3 +50,22 @@ def test_scaled_matrix(ctx, N, scale):
     one.close()
     got.close()
     assert np.linalg.norm(a - b) <= 1e-13 * N * np.linalg.norm(a)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("N,p", [(2, 1), (24, 7), (32, 31), (33, 32), (70, 20), (70, 40), (70, 69)])
+def test_pivot_after_the_first_fails(ctx, N, p, precision):
+    """A = diag(1, .., 1, -1 at p, 1, ..): the factorisation reports pivot p + 1 of whichever block, and the context goes on."""
+    from paper_2501_03061_gb300 import api
+    cell, phi, _ = system(N)
+    d = np.ones(N)
+    d[p] = -1.0
+    dt = np.complex128 if precision == "fp64" else np.complex64
+    shape = (N, 12, 12, 12)
+    W = torch.from_numpy((-d[:, None] * phi).astype(dt).reshape(shape)).cuda()
+    f = torch.from_numpy(phi.astype(dt).reshape(shape)).cuda()
+    with pytest.raises(api.PtimError, match=rf"PT_NOT_PD.*\(pivot {p + 1}\)"):
+        ctx.build_ace_from(W, f, cell=cell, precision=precision)
+    ok = ctx.build_ace_from(-f, f, cell=cell, precision=precision)
+    assert torch.isfinite(torch.view_as_real(ok.xi())).all()
+    ok.close()
