@@ -272,7 +272,8 @@ pt_status pt_overlap(pt_ctx* ctx, const void* A, int N1, const void* B, int N2, 
 /* out_j = sum_k B[k][j] A_k, j < N2: the rotation of an orbital block by an N1 x N2 matrix, e.g.
  * phit = Phi Q into the sigma eigenbasis (Eq. vxdiag) or xi = W L^{-*} of the ACE construction.
  * A: Ng x N1 orbitals, out: Ng x N2 orbitals (device, orbital-major, precision prec; out must
- * not overlap A); B: N1 x N2 complex128 (device, row-major).  Engines as for pt_overlap. */
+ * not overlap A); B: N1 x N2 complex128 (device, row-major).  Engines as for pt_overlap; on CUDA cores
+ * the call uses no workspace of the context. */
 pt_status pt_rotate(pt_ctx* ctx, const void* A, int N1, const void* B, int N2, const pt_grid* grid,
                     pt_precision prec, void* out, void* stream);
 

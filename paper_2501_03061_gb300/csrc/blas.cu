@@ -282,8 +282,7 @@ __global__ void __launch_bounds__(RTHREADS) k_rotate(const cx<T>* __restrict__ A
   }
 }
 
-// FP32 B operand of a rotation, converted once: an FP64 instruction issues every 64 cycles on this part, and
-// every point tile of k_rotate would convert all of B again
+// FP32 B operand of a rotation, converted once
 __global__ void __launch_bounds__(256) k_rot_b32(const c128* __restrict__ B, int ldb, int N1, int N2, c64* __restrict__ out) {
   const int e = blockIdx.x * 256 + threadIdx.x;
   if (e >= N1 * N2) return;
@@ -291,16 +290,22 @@ __global__ void __launch_bounds__(256) k_rot_b32(const c128* __restrict__ B, int
   out[e] = to_cx<float>(B[size_t(k) * ldb + j]);
 }
 
-// The FP32 form of k_rotate: the same tile, the next stage's operands arriving by asynchronous copies, a complex
-// product in two packed instructions (in the order of cfma, so the results are the same bits)
-__global__ void __launch_bounds__(RTHREADS, 3) k_rotate32(const c64* __restrict__ A, const c64* __restrict__ Bm, int N1, int N2,
-                                                       size_t ng, c64 alpha, Epi<float> epi, c64* __restrict__ out) {
+// The FP32 form of k_rotate: the same tile, the next stage's operands on their way during the products of this one, a
+// complex product in two packed instructions (in the order of cfma, so the results are the same bits).
+// BT = c128: B as it is given, each stage of it loaded to registers and converted after the products, so the call needs
+// no workspace.  BT = c64: B from k_rot_b32, by asynchronous copies as A.
+template <class BT>
+__global__ void __launch_bounds__(RTHREADS, 3) k_rotate32(const c64* __restrict__ A, const BT* __restrict__ Bm, int ldb, int N1,
+                                                       int N2, size_t ng, c64 alpha, Epi<float> epi, c64* __restrict__ out) {
+  constexpr bool convert = sizeof(BT) == sizeof(c128);
   __shared__ c64 As[2][KC][RT];
   __shared__ c64 Bs[2][KC][JT];
+  constexpr int BE = (KC * JT) / RTHREADS;  // entries of a B stage per thread
   const size_t r0 = size_t(blockIdx.x) * RT;
   const int j0 = blockIdx.y * JT;
   const int tid = threadIdx.x;
   const int tr = tid % 32, tj = tid / 32;  // 32 x 8
+  BT next[convert ? BE : 1];
   auto fetch = [&](int k0, int buf) {
 #pragma unroll
     for (int pass = 0; pass < (KC * RT) / RTHREADS; ++pass) {
@@ -310,13 +315,24 @@ __global__ void __launch_bounds__(RTHREADS, 3) k_rotate32(const c64* __restrict_
       copy8(&As[buf][kk][r], v ? A + size_t(k0 + kk) * ng + r0 + r : A, v);
     }
 #pragma unroll
-    for (int pass = 0; pass < (KC * JT) / RTHREADS; ++pass) {
+    for (int pass = 0; pass < BE; ++pass) {
       const int e = tid + pass * RTHREADS;
       const int j = e % JT, kk = e / JT;
       const bool v = k0 + kk < N1 && j0 + j < N2;
-      copy8(&Bs[buf][kk][j], v ? Bm + size_t(k0 + kk) * N2 + j0 + j : Bm, v);
+      const BT* src = v ? Bm + size_t(k0 + kk) * ldb + j0 + j : Bm;
+      if constexpr (convert) next[pass] = v ? *src : BT{0, 0};
+      else copy8(&Bs[buf][kk][j], src, v);
     }
     copy_commit();
+  };
+  auto store_b = [&](int buf) {  // the stage in next
+    if constexpr (convert) {
+#pragma unroll
+      for (int pass = 0; pass < BE; ++pass) {
+        const int e = tid + pass * RTHREADS;
+        Bs[buf][e / JT][e % JT] = to_cx<float>(next[pass]);
+      }
+    }
   };
   c64 acc[4][4];
 #pragma unroll
@@ -325,8 +341,10 @@ __global__ void __launch_bounds__(RTHREADS, 3) k_rotate32(const c64* __restrict_
     for (int b = 0; b < 4; ++b) acc[a][b] = czero<float>();
   int buf = 0;
   fetch(0, 0);
+  store_b(0);
   for (int k0 = 0; k0 < N1; k0 += KC, buf ^= 1) {
-    if (k0 + KC < N1) {
+    const bool more = k0 + KC < N1;
+    if (more) {
       fetch(k0 + KC, buf ^ 1);
       copy_wait<1>();
     } else {
@@ -345,6 +363,7 @@ __global__ void __launch_bounds__(RTHREADS, 3) k_rotate32(const c64* __restrict_
         for (int a = 0; a < 4; ++a) acc[a][b] = rl::pfma(bx, av[a].im, rl::pfma(bv, av[a].re, acc[a][b]));
       }
     }
+    if (more) store_b(buf ^ 1);  // last read before the barrier that ended the previous round
     __syncthreads();
   }
 #pragma unroll
@@ -480,7 +499,7 @@ void gram2(pt_ctx* ctx, const cx<T>* A, const cx<T>* B0, c128* C0, const cx<T>* 
 
 template <class T>
 void rotate(pt_ctx* ctx, const cx<T>* A, const c128* Bm, int ldb, int N1, int N2, size_t ng, c128 alpha,
-            const Term* terms, int nterms, cx<T>* out, cudaStream_t st) {
+            const Term* terms, int nterms, cx<T>* out, cudaStream_t st, bool workspace) {
   if constexpr (sizeof(T) == 4) {
     if (ctx->bf16_requested && nterms <= 3) {
       rotate_bf16(ctx, A, Bm, ldb, N1, N2, ng, alpha, terms, nterms, out, st);
@@ -498,9 +517,16 @@ void rotate(pt_ctx* ctx, const cx<T>* A, const c128* Bm, int ldb, int N1, int N2
   }
   dim3 grid(unsigned((ng + RT - 1) / RT), unsigned((N2 + JT - 1) / JT));
   if constexpr (sizeof(T) == 4) {
-    c64* b32 = static_cast<c64*>(ctx->get("rot_b32", size_t(N1) * N2 * sizeof(c64)));
-    PT_LAUNCH(k_rot_b32, (N1 * N2 + 255) / 256, 256, 0, st, Bm, ldb, N1, N2, b32);
-    PT_LAUNCH(k_rotate32, grid, RTHREADS, 0, st, A, b32, N1, N2, ng, to_cx<T>(alpha), epi, out);
+    // Every point tile converts all of B, in instructions that issue every 64 cycles: a launch ahead of it that
+    // converts B once pays from some 128 terms (40^3, 61 x 61 55.7 us without it, 57.7 with; 36^3, 75 x 75 72.2 and 74.1;
+    // 32^3, 150 x 150 151.9 and 149.4; 64^3, 320 x 320 4187 and 4042), but takes workspace of the context.
+    if (N1 <= 128 || !workspace) {
+      PT_LAUNCH(k_rotate32<c128>, grid, RTHREADS, 0, st, A, Bm, ldb, N1, N2, ng, to_cx<T>(alpha), epi, out);
+    } else {
+      c64* b32 = static_cast<c64*>(ctx->get("rot_b32", size_t(N1) * N2 * sizeof(c64)));
+      PT_LAUNCH(k_rot_b32, (N1 * N2 + 255) / 256, 256, 0, st, Bm, ldb, N1, N2, b32);
+      PT_LAUNCH(k_rotate32<c64>, grid, RTHREADS, 0, st, A, b32, N2, N1, N2, ng, to_cx<T>(alpha), epi, out);
+    }
   } else {
     PT_LAUNCH(k_rotate<T>, grid, RTHREADS, 0, st, A, Bm, ldb, N1, N2, ng, to_cx<T>(alpha), epi, out);
   }
@@ -533,9 +559,9 @@ template void gram2<float>(pt_ctx*, const c64*, const c64*, c128*, const c64*, c
 template void gram2<double>(pt_ctx*, const c128*, const c128*, c128*, const c128*, c128*, int, int, size_t, double,
                             cudaStream_t, bool);
 template void rotate<float>(pt_ctx*, const c64*, const c128*, int, int, int, size_t, c128, const Term*, int, c64*,
-                            cudaStream_t);
+                            cudaStream_t, bool);
 template void rotate<double>(pt_ctx*, const c128*, const c128*, int, int, int, size_t, c128, const Term*, int,
-                             c128*, cudaStream_t);
+                             c128*, cudaStream_t, bool);
 template void lincomb<float>(pt_ctx*, c64*, size_t, const Term*, int, cudaStream_t);
 template void lincomb<double>(pt_ctx*, c128*, size_t, const Term*, int, cudaStream_t);
 template void potential_apply<float>(pt_ctx*, c64*, const c64*, const double*, size_t, int, const c64*, double,

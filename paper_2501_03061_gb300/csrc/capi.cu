@@ -424,9 +424,9 @@ pt_status pt_rotate(pt_ctx* ctx, const void* A, int N1, const void* B, int N2, c
     if (prec == PT_FP64)
       pt::rotate<double>(ctx, static_cast<const c128*>(A), Bm, N2, N1, N2, ng, c128{1, 0}, nullptr, 0,
                          static_cast<c128*>(out), st);
-    else
+    else  // on CUDA cores on the caller's buffers alone
       pt::rotate<float>(ctx, static_cast<const c64*>(A), Bm, N2, N1, N2, ng, c128{1, 0}, nullptr, 0,
-                        static_cast<c64*>(out), st);
+                        static_cast<c64*>(out), st, false);
     if (ctx->active_tc || ctx->bf16_requested) pt::gram_tc_check(ctx, st);
     return PT_OK;
   });

@@ -42,7 +42,7 @@ void gram2(pt_ctx* ctx, const cx<T>* A, const cx<T>* B0, c128* C0, const cx<T>* 
            size_t ng, double scale, cudaStream_t st, bool herm = false);
 template <class T>
 void rotate(pt_ctx* ctx, const cx<T>* A, const c128* Bm, int ldb, int N1, int N2, size_t ng, c128 alpha,
-            const Term* terms, int nterms, cx<T>* out, cudaStream_t st);
+            const Term* terms, int nterms, cx<T>* out, cudaStream_t st, bool workspace = true);
 template <class T>
 void lincomb(pt_ctx* ctx, cx<T>* out, size_t n, const Term* terms, int nterms, cudaStream_t st);
 template <class T>
