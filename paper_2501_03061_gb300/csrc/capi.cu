@@ -34,6 +34,7 @@ void* pt_ctx::get(const std::string& name, size_t bytes) {
     cudaFree(it->second.ptr);
     held -= it->second.bytes;
     bufs.erase(it);
+    drop_graphs();
   }
   bytes = std::max<size_t>(bytes, 256);
   if (budget && held + bytes > budget)
@@ -57,7 +58,11 @@ void pt_ctx::release_all() {
   tc_err_clean = false;
   ptim_q_n = 0;
   ptim_warm_valid = false;  // "ptim_xi" is freed
-  // captured graphs hold pointers into the freed workspace
+  drop_graphs();
+}
+
+// captured graphs hold pointers into the workspace: none may outlive a buffer that is freed
+void pt_ctx::drop_graphs() {
   for (auto it = caches.begin(); it != caches.end();) {
     if (it->first.rfind("graph:", 0) == 0) it = caches.erase(it);
     else ++it;

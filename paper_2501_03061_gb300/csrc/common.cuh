@@ -193,6 +193,7 @@ struct pt_ctx {
   // get() of the same name with a larger size, or pt_trim.
   void* get(const std::string& name, size_t bytes);
   void release_all();
+  void drop_graphs();
 };
 
 struct pt_ace {
