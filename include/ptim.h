@@ -361,7 +361,7 @@ typedef struct {
      9 Anderson mixing and residual norms, 10 final Loewdin orthonormalisation,
      11 V_Hxc (midpoint density, Hartree FFT, LDA; params.hxc = 1) */
   double phase_ms[12];
-  int eig_sweeps;           /* Jacobi sweeps of the sigma eigensolves (phase 6) */
+  int eig_sweeps;           /* Jacobi sweeps of the sigma eigensolves (phase 6), FP32 and FP64 ones */
   double total_energy;      /* E(t_n) of the input state (Ha): spin Tr[P_n (-Lap/2 + V_loc)] + E_x
                                (+ E_H + E_xc with params.hxc; the kinetic term carries params.A),
                                from the first iteration, where the midpoint is (Phi_n, sigma_n) */

@@ -278,15 +278,15 @@ __host__ __device__ inline bool jacobi32_done(double off, double off0, double pr
 // One CTA, E and the basis in shared memory (N <= J32_MAX): whole sweeps, two barriers a round (under 1 us at N = 48 against
 // 8.7 us of k_jacobi_round, which is a launch and a chain of FP64 instructions).  A thread for each 2 x 2 block of E, as far
 // as a CTA has them, and its place in E and V without divisions in the rounds (N = 48, the two passes of a solve:
-// 580 -> 445 us).  X: the basis, as FP64.
-constexpr int J32_MAX = 96, J32_THREADS = 1024;
+// 580 -> 445 us).  X: the basis, as FP64; *sweeps_run: the sweeps it took.
+constexpr int J32_MAX = 96, J32_THREADS = 1024, J32_SWEEPS = 12;
 inline int j32_threads(int N) {
   const int half = (N + 1) / 2;
   return std::min(J32_THREADS, std::max(64, (half * half + 31) / 32 * 32));
 }
 constexpr size_t j32_smem(int N) { return 2 * size_t(N) * (N | 1) * sizeof(c64); }
 __global__ void __launch_bounds__(J32_THREADS) k_jacobi32_cta(const c128* __restrict__ A, int N, float floor2,
-                                                              c128* __restrict__ X) {
+                                                              c128* __restrict__ X, double* __restrict__ sweeps_run) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int P = N | 1, Np = N + (N & 1), half = Np / 2;
   c64* a = reinterpret_cast<c64*>(smem_raw);
@@ -305,7 +305,8 @@ __global__ void __launch_bounds__(J32_THREADS) k_jacobi32_cta(const c128* __rest
     v[i * P + j] = c64{i == j ? 1.f : 0.f, 0.f};
   }
   float prev = INFINITY, off0 = 0.f, thr2 = 0.f;
-  for (int sweep = 0; sweep < 12; ++sweep) {
+  int sweep = 0;
+  for (; sweep < J32_SWEEPS; ++sweep) {
     __syncthreads();
     float off = 0.f;
     for (int e = t; e < N * N; e += TH) {
@@ -371,6 +372,7 @@ __global__ void __launch_bounds__(J32_THREADS) k_jacobi32_cta(const c128* __rest
       }
     }
   }
+  if (t == 0) *sweeps_run = sweep;
   __syncthreads();
   for (int e = t; e < N * N; e += TH) {
     const c64 x = v[(e / N) * P + e % N];
@@ -776,7 +778,8 @@ int heev(pt_ctx* ctx, const c128* S, int N, c128* Q, double* d, cudaStream_t st,
   c128* A0 = static_cast<c128*>(ctx->get("heev_A0", size_t(N) * N * sizeof(c128)));
   c128* A1 = static_cast<c128*>(ctx->get("heev_A1", size_t(N) * N * sizeof(c128)));
   c128* V = static_cast<c128*>(ctx->get("heev_V", size_t(N) * N * sizeof(c128)));
-  double* nrm = static_cast<double*>(ctx->get("heev_norm", (2 * OFF_BLOCKS + 2) * sizeof(double)));
+  // the norms, the sweeps of a pass in one CTA, the blocks' sums
+  double* nrm = static_cast<double*>(ctx->get("heev_norm", (2 * OFF_BLOCKS + 3) * sizeof(double)));
   if (Q0) {
     // warm start: rotate into the basis Q0 (Jacobi then starts from a nearly diagonal matrix when
     // Q0 diagonalises a nearby matrix) and accumulate the rotations onto Q0
@@ -789,12 +792,16 @@ int heev(pt_ctx* ctx, const c128* S, int N, c128* Q, double* d, cudaStream_t st,
   }
   const int half = Np / 2;
   dim3 grid((half + JB - 1) / JB, (half + JB - 1) / JB);
-  double h[2] = {0, 0};
+  double h[3] = {0, 0, 0};
+  int sweeps = 0;            // of all passes
+  bool cta_pass = false;     // h[2] will hold a pass's sweeps
   auto norms = [&](auto* A) {
-    PT_LAUNCH_PDL((k_offnorm_part<std::decay_t<decltype(A->re)>>), OFF_BLOCKS, 256, 0, st, A, N, nrm + 2);
-    PT_LAUNCH(k_offnorm_sum, 1, 32, 0, st, nrm + 2, nrm);
+    PT_LAUNCH_PDL((k_offnorm_part<std::decay_t<decltype(A->re)>>), OFF_BLOCKS, 256, 0, st, A, N, nrm + 3);
+    PT_LAUNCH(k_offnorm_sum, 1, 32, 0, st, nrm + 3, nrm);
     PT_CUDA_CHECK(cudaMemcpyAsync(h, nrm, sizeof(h), cudaMemcpyDeviceToHost, st));
     PT_CUDA_CHECK(cudaStreamSynchronize(st));
+    if (cta_pass) sweeps += int(h[2]);
+    cta_pass = false;
     if (!std::isfinite(h[1])) fail(PT_NONFINITE, "non-finite entry in the matrix to diagonalise");
   };
   // Where the caller asks for less than FP64 rounding (rel_tol): FP32 passes on D + E (see k_jacobi32_cta), each basis
@@ -818,7 +825,8 @@ int heev(pt_ctx* ctx, const c128* S, int N, c128* Q, double* d, cudaStream_t st,
         PT_CUDA_CHECK(
             cudaFuncSetAttribute(k_jacobi32_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, int(j32_smem(J32_MAX))));
       });
-      PT_LAUNCH(k_jacobi32_cta, 1, j32_threads(N), j32_smem(N), st, A0, N, float(floor2), X0);
+      PT_LAUNCH(k_jacobi32_cta, 1, j32_threads(N), j32_smem(N), st, A0, N, float(floor2), X0, nrm + 2);
+      cta_pass = true;
     } else {
       // E and V in buffers that are free until the products below
       c64 *e0 = reinterpret_cast<c64*>(G), *e1 = e0 + size_t(N) * N, *v32 = reinterpret_cast<c64*>(X1);
@@ -828,7 +836,7 @@ int heev(pt_ctx* ctx, const c128* S, int N, c128* Q, double* d, cudaStream_t st,
       const double off0 = h[0];
       const float thr2 = float(std::max(1e-15 * off0, floor2) / (double(N) * double(N)));
       double prev = INFINITY;
-      for (int sweep = 0; sweep < 12; ++sweep) {
+      for (int sweep = 0; sweep < J32_SWEEPS; ++sweep) {
         if (sweep > 0) {
           norms(e0);
           if (jacobi32_done(h[0], off0, prev, floor2, N)) break;
@@ -839,6 +847,7 @@ int heev(pt_ctx* ctx, const c128* S, int N, c128* Q, double* d, cudaStream_t st,
           std::swap(e0, e1);
           std::swap(d0, d1);
         }
+        ++sweeps;
       }
       h[0] = off0;
       PT_LAUNCH(k_widen, nb, 256, 0, st, v32, N * N, X0);
@@ -855,7 +864,6 @@ int heev(pt_ctx* ctx, const c128* S, int N, c128* Q, double* d, cudaStream_t st,
     PT_LAUNCH(k_herm_part_and_basis, nb, 256, 0, st, A1, A0, G, V, N);
   }
   double prev_off = INFINITY;
-  int sweeps = 0;
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     norms(A0);
     // Converged when the off-diagonal norm is at the FP64 rounding floor (eps * sqrt(N) * ||A||),
