@@ -302,7 +302,8 @@ pt_status pt_current(pt_ctx* ctx, const void* phi, const void* sigma, int N, con
  * matrix P = Phi sigma Phi^* (Sec. II-A, Eq. mix_P).  phi: Ng x N orbital-major, precision prec
  * (16-byte aligned); sigma: N x N complex128 row-major (Hermitian); rho: Ng doubles.  All device
  * pointers.  The FP32 forms form chi = Phi sigma with the library's rotation (tensor cores when
- * enabled) and sum the products in FP64.  Workspace: one Ng x N block held by the context. */
+ * enabled) and sum the products to 48 bits or more (in FP64 where a sum leaves the FP32 range).
+ * Workspace: one Ng x N block held by the context. */
 pt_status pt_density(pt_ctx* ctx, const void* phi, const void* sigma, int N, const pt_grid* grid, pt_precision prec,
                      double spin, double* rho, void* stream);
 

@@ -70,31 +70,44 @@ struct RunSum {
       s = n;
     }
   }
-  // an overflowed sum is itself (its error term is not a number)
-  __device__ __forceinline__ double value() const { return isfinite(s) ? double(s) + double(e) : double(s); }
+  __device__ __forceinline__ double value() const { return double(s) + double(e); }
 };
+
+// the terms of orbitals j, j + 1, ... to the four sums in turn
+template <class T, class Sum>
+__device__ __forceinline__ double density_sum(const cx<T>* __restrict__ chi, const cx<T>* __restrict__ phi, int N, size_t ng,
+                                              size_t r, bool& finite) {
+  Sum acc[4];
+  int j = 0;
+  for (; j + 4 <= N; j += 4) {
+    cx<T> a[4], b[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      a[u] = chi[size_t(j + u) * ng + r];
+      b[u] = phi[size_t(j + u) * ng + r];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[u].add(a[u].re * b[u].re + a[u].im * b[u].im);
+  }
+  for (; j < N; ++j) {
+    const cx<T> a = chi[size_t(j) * ng + r], b = phi[size_t(j) * ng + r];
+    acc[0].add(a.re * b.re + a.im * b.im);
+  }
+  finite = true;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) finite = finite && isfinite(acc[u].s + acc[u].e);
+  return (acc[0].value() + acc[1].value()) + (acc[2].value() + acc[3].value());
+}
 
 template <class T>
 __global__ void __launch_bounds__(256) k_density(const cx<T>* __restrict__ chi, const cx<T>* __restrict__ phi, int N,
                                                  size_t ng, double spin, double* __restrict__ rho) {
   for (size_t r = size_t(blockIdx.x) * blockDim.x + threadIdx.x; r < ng; r += size_t(gridDim.x) * blockDim.x) {
-    RunSum<T> acc[4];
-    int j = 0;
-    for (; j + 4 <= N; j += 4) {
-      cx<T> a[4], b[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        a[u] = chi[size_t(j + u) * ng + r];
-        b[u] = phi[size_t(j + u) * ng + r];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) acc[u].add(a[u].re * b[u].re + a[u].im * b[u].im);
-    }
-    for (; j < N; ++j) {
-      const cx<T> a = chi[size_t(j) * ng + r], b = phi[size_t(j) * ng + r];
-      acc[0].add(a.re * b.re + a.im * b.im);
-    }
-    rho[r] = spin * ((acc[0].value() + acc[1].value()) + (acc[2].value() + acc[3].value()));
+    bool finite;
+    double sum = density_sum<T, RunSum<T>>(chi, phi, N, ng, r, finite);
+    // a sum that left the FP32 range, or met a term that is not finite, is taken in FP64
+    if (sizeof(T) == 4 && !finite) sum = density_sum<T, RunSum<double>>(chi, phi, N, ng, r, finite);
+    rho[r] = spin * sum;
   }
 }
 
