@@ -192,6 +192,7 @@ struct pt_ctx {
   // Grow-only named workspace.  The returned pointer stays valid until the next
   // get() of the same name with a larger size, or pt_trim.
   void* get(const std::string& name, size_t bytes);
+  bool fits(const std::string& name, size_t bytes) const;  // the HBM budget allows get(name, bytes)
   void release_all();
   void drop_graphs();
 };

@@ -143,9 +143,16 @@ long long exchange_lines(pt_ctx* ctx, const c64* src, const double* occ, int N, 
   std::swap(gt.L[0], gt.L[1]);
   const float* kt = static_cast<const float*>(kernel_table(ctx, gt, k, PT_FP32));
   // as few tiles as the side allows, all of about the same size (36^3 N = 75: 25 + 25 + 25 instead of 37 + 37 + 1)
-  const int nb = (N + B - 1) / B, mb = (M + B - 1) / B;
+  int nb = (N + B - 1) / B, mb = (M + B - 1) / B;
+  const std::string name = ctx->tagged("exchange_scratch");
+  // A symmetric tile has a field for each of its N^2 slots, though its pairs fill N (N + 1)/2 of them: slots of the triangle
+  // alone cost every pass (24^3 N = 16 24.5 -> 25.6 us, 64^3 N = 320 105.5 -> 106.9 ms).  Where the context's HBM budget
+  // has no room for them, two tiles a side run in the triangle's.
+  const bool tight = sym && nb == 1 && N > 1 && !ctx->fits(name, size_t(N) * N * field);
+  if (tight) nb = mb = 2;
   const int bi = (N + nb - 1) / nb, bj = (M + mb - 1) / mb;
-  c64* scratch = static_cast<c64*>(ctx->get(ctx->tagged("exchange_scratch"), size_t(bi) * bj * field));
+  const size_t slots = tight ? size_t(N) * (N + 1) / 2 : size_t(bi) * bj;
+  c64* scratch = static_cast<c64*>(ctx->get(name, slots * field));
   for (int J = 0; J * bj < M; ++J)
     for (int I = 0; sym ? I <= J : I * bi < N; ++I) {
       const Tile t{I * bi, std::min(bi, N - I * bi), J * bj, std::min(bj, M - J * bj), int(sym), int(sym && I == J), int(I == 0)};
