@@ -451,17 +451,28 @@ void gram(pt_ctx* ctx, const cx<T>* A, const cx<T>* B, int N1, int N2, size_t ng
     }
   }
   const bool f32 = sizeof(T) == 4;
-  // FP32 tile of 64, 48 or 32 orbitals: the one that pads N1 x N2 least (75 x 75 in four tiles of 48 instead of 64: 145 ->
-  // 85 us), the larger where they tie: it reads less per product
+  herm = herm && (N1 == N2);
+  // FP32 tile of 64 orbitals, or of 48 or 32 where that pads less: the one whose CTAs are done first.  A CTA takes 1, 0.58 or
+  // 0.35 units a point (a smaller tile reads more per product) and 80 points' worth to start and to write its sums; an
+  // SM runs its share of CTAs, one more of the smallest where the idle ones below the diagonal leave the others
+  // unevenly spread.  Measured, Hermitian, in tiles of 32 / 48 / 64: 32^3 N = 200 365 / 227 / 258 us (32 pads least),
+  // N = 400 1172 / 704 / 712, N = 600 3482 / 1389 / 1397, 36^3 N = 75 115 / 77 / 121, 16^3 N = 40 21 / 23 / 29.
   int R = 4;
   if (f32) {
-    auto area = [&](int r) { return size_t((N1 + 16 * r - 1) / (16 * r)) * ((N2 + 16 * r - 1) / (16 * r)) * r * r; };
+    auto side = [&](int n, int r) { return (long long)(n + 16 * r - 1) / (16 * r); };
+    auto padded = [&](int r) { return side(N1, r) * side(N2, r) * r * r; };
+    auto cost = [&](int r) {
+      const long long sms = ctx->num_sms, ti = side(N1, r), tj = side(N2, r);
+      const long long tiles = herm ? ti * (ti + 1) / 2 : ti * tj, splits = std::max(1ll, 2 * sms / tiles);
+      const long long chunk = ((ng + splits - 1) / splits + G4K - 1) / G4K * G4K;
+      const long long turns = (tiles * ((ng + chunk - 1) / chunk) + sms - 1) / sms + (r == 2 && herm && ti > 1);
+      return double(turns * (chunk + 80)) * (r == 4 ? 1.0 : r == 3 ? 0.58 : 0.35);
+    };
     for (int r = 3; r >= 2; --r)
-      if (area(r) < area(R)) R = r;
+      if (padded(r) < padded(4) && cost(r) < cost(R)) R = r;
   }
   const int tile = f32 ? 16 * R : GT;
   const int kstep = f32 ? G4K : GK;
-  herm = herm && (N1 == N2);
   const int ti = (N1 + tile - 1) / tile, tj = (N2 + tile - 1) / tile;
   const int tiles = herm ? ti * (ti + 1) / 2 : ti * tj;
   // enough splits along r to fill the GPU about four times; twice, one wave of the two CTAs per SM, for the FP32 tile
