@@ -11,7 +11,9 @@
 // back, and the last x pass evaluates the LDA point by point, adds V_loc and writes the total local potential.
 // Small tiles (4 x lines, 8 columns) give every pass 2-4 CTAs per SM: FP64 issues at 1/64 rate, so a pass
 // on nz of the 152 SMs is bound by that many FP64 pipes.  60^3: 114 us against 303 us of whole-plane tiles on the
-// full spectrum, of which the LDA's transcendentals took 100.
+// full spectrum, of which the LDA's transcendentals took 100.  The passes are dependent launches, each reading its
+// twiddles while the one before drains: five launches in a row cost small grids more than the three of the whole planes
+// (5^3 33 -> 37 us, 60 x 3 x 4 38 -> 48), as dependent ones 29 and 39 (16^3 54 -> 45, 36^3 74 -> 66).
 #include <algorithm>
 
 #include "fft.cuh"
@@ -119,6 +121,7 @@ __global__ void __launch_bounds__(NT) k_hxc_x_fwd(GridPlan gp, const double* __r
   const int z = blockIdx.y, nx = gp.nx, ny = gp.ny, hx = nx / 2 + 1, pitch = gp.pitch_x;
   const int y0 = blockIdx.x * XL * 2;
   for (int t = threadIdx.x; t < nx; t += NT) tw[t] = twg[t];
+  pdl_launch_dependents();
   const double* f = rho + (size_t(z) * ny + y0) * nx;
   for (int e = threadIdx.x; e < XL * nx; e += NT) {
     const int l = e / nx, x = e - l * nx, y = y0 + 2 * l;
@@ -143,6 +146,8 @@ __global__ void __launch_bounds__(NT) k_hxc_y(GridPlan gp, c128* __restrict__ ha
   __shared__ c128 buf[CP * kMaxDim];
   const int ny = gp.ny, hx = gp.nx / 2 + 1, k0 = blockIdx.x * CL, cols = min(CL, hx - k0);
   for (int t = threadIdx.x; t < ny; t += NT) tw[t] = twg[gp.nx + t];
+  pdl_wait();  // the pass before
+  pdl_launch_dependents();
   c128* f = half + size_t(blockIdx.y) * ny * hx + k0;
   for (int e = threadIdx.x; e < CL * ny; e += NT) {
     const int y = e / CL, c = e % CL;
@@ -164,6 +169,8 @@ __global__ void __launch_bounds__(NT) k_hxc_z(GridPlan gp, c128* __restrict__ ha
   const int nx = gp.nx, ny = gp.ny, nz = gp.nz, hx = nx / 2 + 1, y = blockIdx.y;
   const int k0 = blockIdx.x * CL, cols = min(CL, hx - k0);
   for (int t = threadIdx.x; t < nz; t += NT) tw[t] = twg[nx + ny + t];
+  pdl_wait();  // the pass before
+  pdl_launch_dependents();
   c128* f = half + size_t(y) * hx + k0;
   for (int e = threadIdx.x; e < CL * nz; e += NT) {
     const int z = e / CL, c = e % CL;
@@ -195,6 +202,8 @@ __global__ void __launch_bounds__(NT) k_hxc_x_inv(GridPlan gp, const c128* __res
   const int z = blockIdx.y, nx = gp.nx, ny = gp.ny, hx = nx / 2 + 1, pitch = gp.pitch_x;
   const int y0 = blockIdx.x * XL * 2;
   for (int t = threadIdx.x; t < nx; t += NT) tw[t] = twg[t];
+  pdl_wait();  // the pass before
+  pdl_launch_dependents();
   const c128* f = half + (size_t(z) * ny + y0) * hx;
   for (int e = threadIdx.x; e < XL * hx; e += NT) {
     const int l = e / hx, k = e - l * hx, y = y0 + 2 * l;
@@ -272,10 +281,10 @@ void hxc_potential(pt_ctx* ctx, const double* rho, const double* vloc, const pt_
   double* sums = part ? reinterpret_cast<double*>(half + nh) : nullptr;
   const c128* tw = static_cast<const c128*>(ft.tw);
   PT_LAUNCH(k_hxc_x_fwd, dim3(xc, g.nz), NT, 0, st, ft.plan, rho, half, tw);
-  PT_LAUNCH(k_hxc_y<false>, dim3(cc, g.nz), NT, 0, st, ft.plan, half, tw);
-  PT_LAUNCH(k_hxc_z, dim3(cc, g.ny), NT, 0, st, ft.plan, half, static_cast<const double*>(ft.g2d), 1.0 / double(ng), tw);
-  PT_LAUNCH(k_hxc_y<true>, dim3(cc, g.nz), NT, 0, st, ft.plan, half, tw);
-  PT_LAUNCH(k_hxc_x_inv, dim3(xc, g.nz), NT, 0, st, ft.plan, half, rho, vloc, v, sums, tw);
+  PT_LAUNCH_PDL(k_hxc_y<false>, dim3(cc, g.nz), NT, 0, st, ft.plan, half, tw);
+  PT_LAUNCH_PDL(k_hxc_z, dim3(cc, g.ny), NT, 0, st, ft.plan, half, static_cast<const double*>(ft.g2d), 1.0 / double(ng), tw);
+  PT_LAUNCH_PDL(k_hxc_y<true>, dim3(cc, g.nz), NT, 0, st, ft.plan, half, tw);
+  PT_LAUNCH_PDL(k_hxc_x_inv, dim3(xc, g.nz), NT, 0, st, ft.plan, half, rho, vloc, v, sums, tw);
   if (part) PT_LAUNCH(k_hxc_energy, (2 * g.nz + 127) / 128, 128, 0, st, sums, xc, g.nz, part);
 }
 
