@@ -10,7 +10,7 @@
 // one complex x line, y and z lines run on nx/2 + 1 columns, the z pass applies 4 pi/|G|^2 / Ng and transforms
 // back, and the last x pass evaluates the LDA point by point, adds V_loc and writes the total local potential.
 // Small tiles (4 x lines, 8 columns) give every pass 2-4 CTAs per SM: FP64 issues at 1/64 rate, so a pass
-// on nz of the 152 SMs is bound by that many FP64 pipes.  60^3: 114 us against 303 us of whole-plane tiles on the
+// on nz of the 152 SMs is bound by that many FP64 pipes.  60^3: 123 us against 331 us of whole-plane tiles on the
 // full spectrum, of which the LDA's transcendentals took 100.  The passes are dependent launches, each reading its
 // twiddles while the one before drains: five launches in a row cost small grids more than the three of the whole planes
 // (5^3 33 -> 37 us, 60 x 3 x 4 38 -> 48), as dependent ones 29 and 39 (16^3 54 -> 45, 36^3 74 -> 66).
@@ -280,11 +280,21 @@ void hxc_potential(pt_ctx* ctx, const double* rho, const double* vloc, const pt_
   c128* half = static_cast<c128*>(ctx->get("hxc_scratch", nh * sizeof(c128) + 2 * size_t(xc) * g.nz * sizeof(double)));
   double* sums = part ? reinterpret_cast<double*>(half + nh) : nullptr;
   const c128* tw = static_cast<const c128*>(ft.tw);
+  // Launched dependent, the CTAs of a pass settle where the pass before leaves room.  With more than two a SM in both of two
+  // passes that leaves some SMs with twice the work of others (64^3 130 -> 158 us; 64 x 60 x 60, 300 CTAs a pass, 129
+  // -> 121): those run one after another.
+  const int two = 2 * ctx->num_sms;
+  const bool crowded = cc * g.ny > two && cc * g.nz > two;
+  auto next = [&](auto kernel, dim3 grid, auto... args) {
+    if (crowded) PT_LAUNCH(kernel, grid, NT, 0, st, args...);
+    else PT_LAUNCH_PDL(kernel, grid, NT, 0, st, args...);
+  };
+  const double* g2 = static_cast<const double*>(ft.g2d);
   PT_LAUNCH(k_hxc_x_fwd, dim3(xc, g.nz), NT, 0, st, ft.plan, rho, half, tw);
-  PT_LAUNCH_PDL(k_hxc_y<false>, dim3(cc, g.nz), NT, 0, st, ft.plan, half, tw);
-  PT_LAUNCH_PDL(k_hxc_z, dim3(cc, g.ny), NT, 0, st, ft.plan, half, static_cast<const double*>(ft.g2d), 1.0 / double(ng), tw);
-  PT_LAUNCH_PDL(k_hxc_y<true>, dim3(cc, g.nz), NT, 0, st, ft.plan, half, tw);
-  PT_LAUNCH_PDL(k_hxc_x_inv, dim3(xc, g.nz), NT, 0, st, ft.plan, half, rho, vloc, v, sums, tw);
+  next(k_hxc_y<false>, dim3(cc, g.nz), ft.plan, half, tw);
+  next(k_hxc_z, dim3(cc, g.ny), ft.plan, half, g2, 1.0 / double(ng), tw);
+  next(k_hxc_y<true>, dim3(cc, g.nz), ft.plan, half, tw);
+  next(k_hxc_x_inv, dim3(xc, g.nz), ft.plan, half, rho, vloc, v, sums, tw);
   if (part) PT_LAUNCH(k_hxc_energy, (2 * g.nz + 127) / 128, 128, 0, st, sums, xc, g.nz, part);
 }
 

@@ -8,7 +8,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("shape", [(5, 5, 5), (60, 3, 4), (24, 20, 18)])
+@pytest.mark.parametrize("shape", [(5, 5, 5), (60, 3, 4), (24, 20, 18), (64, 64, 32), (64, 64, 64)])
 def test_captured_and_back_to_back(shape):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
