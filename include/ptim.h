@@ -148,8 +148,8 @@ pt_status pt_trim(pt_ctx* ctx);
  *                    cost per pair falls with the pair tile even past L2 residency, 24^3 with 64
  *                    orbitals 0.47 -> 0.22 ms from 48 MiB to 512 MiB; smaller values give more,
  *                    smaller batches).
- *   "exchange64_scratch_bytes"  the same for the 64^3 FP32 exchange (default 512 MiB: 16 x 16 pair
- *                    tiles).
+ *   "exchange64_scratch_bytes"  the same for the 64^3 FP32 exchange of single calls (default 512 MiB:
+ *                    16 x 16 pair tiles; a batched call takes "scratch_bytes" on every grid).
  *   "tc_gram"        1: in the PT_FP32 form, run the Gram contractions (A^H B over the grid) on
  *                    the tensor cores with a 3-product TF32 split (hi*hi + hi*lo + lo*hi) that
  *                    keeps FP32-level accuracy; 0 (default): CUDA cores.
@@ -224,10 +224,12 @@ typedef struct {
 
 /* Batched exchange: `count` independent V_x applications (different orbital counts, grids and
  * kernels) in one call, in the given precision, in item order on `stream`.  Where the pair-tile
- * size matters (FP64 and orthorhombic grids) it is chosen by timing a few candidates the first time
- * the grid is seen (option "autotune", default 1).  The first call with a given item set (the same buffers and sizes)
+ * size matters (FP64, and FP32 grids with an axis below 16 points) it is chosen by timing a few
+ * candidates the first time the grid is seen (option "autotune", default 1); FP32 items of other
+ * grids take "scratch_bytes".  The first call with a given item set (the same buffers and sizes)
  * runs eagerly and records the batch into a CUDA graph; later calls with the same item set
- * replay the graph as one launch (option "graphs", default 1).  pt_trim drops the graphs.
+ * replay the graph as one launch (option "graphs", default 1).  pt_trim drops the graphs, and so
+ * does any call that replaces a workspace buffer by a larger one: the batch is then recorded anew.
  * Synchronises `stream` once at the end to read the kernels' error word (PT_TIMEOUT if a
  * bounded wait expired).  *pair_ffts (optional) receives the pair FFTs of the batch and
  * *graph_nodes (optional) the node count of the graph that ran (0: eager).  No counterpart

@@ -3,14 +3,16 @@
 // Eq. vxdiag, applied per instance).
 //
 // Host runtime around the exchange kernels:
-//   * autotuner: on the grids whose cost depends on it (FP64, orthorhombic cells) the pair-tile size
-//     (how many pair fields one FFT batch holds, which sets the L2 footprint and the launch count) is
+//   * autotuner: on the grids whose cost depends on it (FP64, and FP32 with an axis below 16 points) the pair-tile
+//     size (how many pair fields one FFT batch holds, which sets the L2 footprint and the launch count) is
 //     picked by timing candidates (budgets of 12 MiB to 512 MiB) on the first item of that grid (its
-//     first min(N, 32) orbitals) and kept in the context; the FP32 line kernels of cubic grids take the
+//     first min(N, 32) orbitals) and kept in the context; the FP32 line kernels take the
 //     largest tile, which was the fastest on every side (24^3 N = 64: 0.22 ms with 512 MiB, 0.47 with 48);
 //   * concurrent branches: items are dealt to `batch_streams` streams (longest first, by pair
 //     FFTs x grid points), each with its own scratch buffers, forked from and joined back to the
-//     caller's stream with events, so the small items' kernels fill the tails of the large ones';
+//     caller's stream with events, so the small items' kernels fill the tails of the large ones' (the FP32
+//     line kernels gain nothing by it: 64 instances 0.71 s on four branches, 0.63 on one, because concurrent items
+//     evict one another's pair fields from L2; the default is that of the kernels before them);
 //   * CUDA graphs: the first call with a given item set runs eagerly once (this sizes every
 //     workspace, builds schedules and tables and encodes nothing that later changes), then the
 //     whole batch is captured on a context-owned stream into one graph, which this and every

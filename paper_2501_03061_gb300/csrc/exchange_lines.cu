@@ -15,7 +15,7 @@
 // less than the write and the two reads of v_ij that it saves.
 //
 // What bounds it: registers.  A 64-point line is 128 registers, so an SM holds 12 warps (N <= 32: 20),
-// and the passes run at 25-45% of the issue rate, 30-55% of the L1 rate and, at 64^3, 4.2-5.2 TB/s of memory
+// and the passes run at 25-45% of the issue rate, 35-60% of the L1 rate and, at 64^3, 4.2-5.2 TB/s of memory
 // (0.63-0.78 of a copy), waiting on the loads
 // and stores of lines between the transforms.  Measured on GB300, one V_x application, all pairs
 // symmetric (this form against the tile kernels, at 64 against the TMA pipeline it replaced):

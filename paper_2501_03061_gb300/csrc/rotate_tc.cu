@@ -25,8 +25,8 @@
 // ring of their own, so that their 32 KB copies run ahead of the conversions (with one ring of two for both
 // operands a stage's buffers took the MMAs, the copy and the conversion in turn; 54^3, 200 x 200 512 -> 446 us, 60^3,
 // 150 x 150 434 -> 361, 64^3, 320 x 320 1371 -> 1266), and A operands in TMEM in place of swizzled rows in shared memory
-// take a third off the traffic of its pipe (446 -> 419, 361 -> 345, 1266 -> 1198).  A stage takes about 1900 cycles, of
-// which the MMAs are 770; 48 KB of operands come in for each at 48 GB/s a CTA.  Two converter warpgroups at 96
+// take a third off the traffic of its pipe (446 -> 419, 361 -> 345, 1266 -> 1198).  A stage takes 1620 cycles
+// (1880 at the benchmark's clock), of which the MMAs are 770; its 48 KB of operands come in at 53 GB/s a CTA.  Two converter warpgroups at 96
 // registers a thread ran slower (507 us), and so did two row tiles that share the B' stages (501): the
 // epilogue of both at once leaves the MMAs without a free accumulator, it seems, for longer than the loads saved.
 //   CTAs are persistent and walk the tiles with a grid stride; the two TMEM accumulators alternate between periods, so the
