@@ -50,10 +50,10 @@ void* pt_ctx::get(const std::string& name, size_t bytes) {
   return p;
 }
 
-bool pt_ctx::fits(const std::string& name, size_t bytes) const {
+bool pt_ctx::fits(const std::string& name, size_t bytes, size_t more) const {
   const auto it = bufs.find(name);
   const size_t own = it == bufs.end() ? 0 : it->second.bytes;
-  return !budget || own >= bytes || held - own + std::max<size_t>(bytes, 256) <= budget;
+  return !budget || own >= bytes || held - own + bytes + more <= budget;
 }
 
 void pt_ctx::release_all() {

@@ -192,7 +192,8 @@ struct pt_ctx {
   // Grow-only named workspace.  The returned pointer stays valid until the next
   // get() of the same name with a larger size, or pt_trim.
   void* get(const std::string& name, size_t bytes);
-  bool fits(const std::string& name, size_t bytes) const;  // the HBM budget allows get(name, bytes)
+  // the buffer holds so much already, or the HBM budget allows get(name, bytes) and `more` bytes beside it
+  bool fits(const std::string& name, size_t bytes, size_t more) const;
   void release_all();
   void drop_graphs();
 };

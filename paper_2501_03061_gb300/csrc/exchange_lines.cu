@@ -147,8 +147,9 @@ long long exchange_lines(pt_ctx* ctx, const c64* src, const double* occ, int N, 
   const std::string name = ctx->tagged("exchange_scratch");
   // A symmetric tile has a field for each of its N^2 slots, though its pairs fill N (N + 1)/2 of them: slots of the triangle
   // alone cost every pass (24^3 N = 16 24.5 -> 25.6 us, 64^3 N = 320 105.5 -> 106.9 ms).  Where the context's HBM budget
-  // has no room for them, two tiles a side run in the triangle's.
-  const bool tight = sym && nb == 1 && N > 1 && !ctx->fits(name, size_t(N) * N * field);
+  // has no room for them and for those of a batch's other branches, two tiles a side run in the triangle's.
+  const size_t branches = size_t(1 + ctx->batch_streams) * (budget / 2);
+  const bool tight = sym && nb == 1 && N > 1 && !ctx->fits(name, size_t(N) * N * field, branches);
   if (tight) nb = mb = 2;
   const int bi = (N + nb - 1) / nb, bj = (M + mb - 1) / mb;
   const size_t slots = tight ? size_t(N) * (N + 1) / 2 : size_t(bi) * bj;

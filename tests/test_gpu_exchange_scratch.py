@@ -43,3 +43,28 @@ def test_budget_of_one_field_per_pair(n, nz, N):
         assert torch.linalg.norm(out - ref) <= 1e-6 * torch.linalg.norm(ref)
     with pytest.raises(api.PtimError, match="PT_OOM"):
         run(pairs - 4096)
+
+
+def test_budget_of_a_batch():
+    """Four branches, each with the fields of its largest item's pairs: every branch finds its room."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2501_03061_gb300 import api
+    rng = np.random.default_rng(8)
+    calls, pairs = [], 0
+    for n, N in ((24, 40), (30, 30), (32, 28), (20, 50)):
+        src = torch.from_numpy((rng.standard_normal((N, n, n, n)) + 1j * rng.standard_normal((N, n, n, n))).astype(np.complex64)).cuda()
+        calls.append({"src": src, "occ": torch.linspace(1, 0.1, N, dtype=torch.float64).cuda(), "cell": synth.cubic(n, 0.3 * n),
+                      "kernel": KERNEL, "out": torch.empty_like(src)})
+        pairs += N * (N + 1) // 2 * n ** 3 * 8
+    got = []
+    for budget in (0, pairs + (64 << 10)):
+        ctx = api.Context(0, budget)
+        try:
+            for _ in range(2):
+                outs = ctx.apply_exchange_batched(calls, precision="fp32")[0]
+            got.append([o.clone() for o in outs])
+        finally:
+            ctx.close()
+    for a, b in zip(*got):
+        assert torch.linalg.norm(a - b) <= 1e-6 * torch.linalg.norm(a)
